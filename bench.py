@@ -48,7 +48,7 @@ REF_BUDGET_S = 120.0
 # of one launch of a sweep kernel, with the hash of the kernel sources it was
 # captured on: a figure is reported only while the sources still hash the same
 # (a changed kernel has no traffic figure until it is captured again).
-KERNEL_SOURCES = ("paper_1103_4887_gb300/csrc/sweep.cu", "paper_1103_4887_gb300/csrc/device.cuh",
+KERNEL_SOURCES = ("paper_1103_4887_gb300/csrc/sweep.cu", "paper_1103_4887_gb300/csrc/device.cuh", "paper_1103_4887_gb300/csrc/fixed.cuh",
                   "paper_1103_4887_gb300/csrc/scheme.cuh", "paper_1103_4887_gb300/csrc/stats.cuh",
                   "paper_1103_4887_gb300/csrc/internal.h")
 TRAFFIC = {

@@ -22,7 +22,7 @@ CHECKED_SOURCES = ["sweep.cu"]  # the translation units that differ under PIMC_C
 ROOT = os.path.dirname(HERE)
 
 CU_SOURCES = ["sweep.cu", "ops.cu", "runtime.cu", "noalloc.cu", "hmc.cu"]
-HEADERS = ["device.cuh", "internal.h", "stats.cuh", "scheme.cuh", "reduce.cuh"]
+HEADERS = ["device.cuh", "fixed.cuh", "internal.h", "stats.cuh", "scheme.cuh", "reduce.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -8,6 +8,8 @@
 #include <type_traits>
 #include <cuda_runtime.h>
 
+#include "fixed.cuh"
+
 namespace pimc {
 
 constexpr int kMaxD = 4;
@@ -59,14 +61,10 @@ template <> struct Num<double> {
     static __device__ __forceinline__ double exm1(double x) { return expm1(x); }
     static __device__ __forceinline__ double div(double a, double b) { return a / b; }
     static __device__ __forceinline__ double uni(uint32_t hi, uint32_t lo) { return u01d(hi, lo); }
-    // Box-Muller: r cos(2 pi u2), r sin(2 pi u2), r = sqrt(-2 log u1)
+    // Box-Muller: r cos(2 pi u2), r sin(2 pi u2), r = sqrt(-2 log u1), in fixed point
     static __device__ __forceinline__ void box_muller(uint4 w, double& z0, double& z1)
     {
-        const double r = sqrt(-2.0 * log(u01d(w.x, w.y)));
-        double s, c;
-        sincospi(2.0 * u01d(w.z, w.w), &s, &c);
-        z0 = r * c;
-        z1 = r * s;
+        fx_box_muller(w.x, w.y, w.z, w.w, z0, z1);
     }
     static constexpr double psi_cut = 1e-6;
     static constexpr double dpsi_cut = 1e-3;
@@ -644,6 +642,32 @@ __device__ __forceinline__ void rk4_map(const R* x, const R* p, R I, R dt, R* f)
     for (int a = 0; a < D; ++a) f[a] = x[a] + dt / R(6) * (acc[a] + k[a]);
 }
 
+// The FP64 HH map outside the range of the fixed-point one (rare: one copy, called).
+static __device__ __noinline__ void hh_map_fp64(const double* x, const double* p, double I, double dt, double* f)
+{
+    rk4_map<HH<double>, double>(x, p, I, dt, f);
+}
+
+// The map f as every kernel evaluates it: the FP64 HH map in 64-bit fixed point (fixed.cuh; fx holds the step's
+// constants) where its range allows, else rk4_map.
+template <class Model, class R>
+__device__ __forceinline__ void map_step(const HhFixed& fx, const R* x, const R* p, R I, R dt, R* f)
+{
+    if constexpr (std::is_same<Model, HH<double>>::value) {
+        const HhFixedParams q = hh_fixed_params(fx, p, dt);
+        if (!hh_map_fixed(fx, q, x, I, f)) {
+            double xx[4] = {x[0], x[1], x[2], x[3]}, pp[kMaxP], ff[4];
+#pragma unroll
+            for (int l = 0; l < kMaxP; ++l) pp[l] = p[l];
+            hh_map_fp64(xx, pp, I, dt, ff);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) f[a] = ff[a];
+        }
+    } else {
+        rk4_map<Model, R>(x, p, I, dt, f);
+    }
+}
+
 // Reverse mode through the RK4 step: the stage states are recomputed from x
 // (nothing stored); once f = f(x) is formed, cot(f, w) fills the cotangent w
 // of f (e.g. from the residual x_{n+1} - f), which is then pulled back stage
@@ -705,9 +729,13 @@ template <class R> __device__ __forceinline__ R sqdiff(R Rw, R dp, R d)
 
 // Metropolis rule written with E = -log(u), which can be formed before dA is
 // known: u < exp(-dA) <=> dA < E (and dA <= 0 < E); NaN compares false.
-template <class R> __device__ __forceinline__ R neglog(R u);
-template <> __device__ __forceinline__ double neglog<double>(double u) { return -log(u); }
-template <> __device__ __forceinline__ float neglog<float>(float u) { return -__logf(u); }
+// From the two Philox words of u.
+template <class R> __device__ __forceinline__ R neglog_uniform(uint32_t hi, uint32_t lo);
+template <> __device__ __forceinline__ double neglog_uniform<double>(uint32_t hi, uint32_t lo)
+{
+    return fx_neglog_uniform(hi, lo);
+}
+template <> __device__ __forceinline__ float neglog_uniform<float>(uint32_t hi, uint32_t) { return -__logf(u01f(hi)); }
 
 // Metropolis rule, Eq. (Paccept): accept iff dA <= 0 or u < exp(-dA);
 // a non-finite dA is a rejection.

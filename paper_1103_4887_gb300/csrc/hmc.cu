@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kBlock) hmc_begin_kernel(Ctx c, HmcScalars* hs
     grid_sums_last_block<1>(c, v, k0, wsum, &last);
     if (last && threadIdx.x == 0) {
         hs->K0 = k0[0];
-        hs->E = -log(u01d(wacc.x, wacc.y));
+        hs->E = fx_neglog_uniform(wacc.x, wacc.y);
         hs->eps = eps_t;
         hs->oob = 0;
         hs->accept = 0;  // set by the last leapfrog step

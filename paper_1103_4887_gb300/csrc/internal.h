@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "fixed.cuh"
+
 namespace pimc {
 
 constexpr int kBlock = 128;          // threads per CTA of the whole-path kernels
@@ -69,6 +71,7 @@ struct Ctx {
     int64_t wait_ns;
     int skip_cta;
     int64_t tile;                 // sites per CTA in the sweep kernel
+    HhFixed fx;                   // constants of dt of the fixed-point FP64 HH map
     unsigned* chk;                // [3][ldx] site visits (even phase, odd phase, parameter-move cache
                                   // writes), then a u64 count of executed parameter moves: counted by
                                   // builds compiled with PIMC_CHECK only

@@ -29,7 +29,7 @@ static __device__ __align__(256) unsigned char g_action_scratch[kScratchBytes];
 
 template <class Model>
 __global__ void __launch_bounds__(kStaticBlock)
-action_static_kernel(int64_t M, double dt, double Rm, double Rf0, double Rf1, double Rf2, double Rf3,
+action_static_kernel(HhFixed fx, int64_t M, double dt, double Rm, double Rf0, double Rf1, double Rf2, double Rf3,
                      const double* X, const double* p, const double* y, const double* I, double* out,
                      unsigned char* scratch)
 {
@@ -52,7 +52,7 @@ action_static_kernel(int64_t M, double dt, double Rm, double Rf0, double Rf1, do
         }
         if (n < M) {
             double f[D];
-            rk4_map<Model, double>(x, q, I[n], dt, f);
+            map_step<Model, double>(fx, x, q, I[n], dt, f);
             for (int a = 0; a < D; ++a) {
                 const double e = X[a * (M + 1) + n + 1] - f[a];
                 v[1] += 0.5 * Rf[a] * e * e;
@@ -152,13 +152,13 @@ extern "C" int pimc_action_static(int model, int64_t M, double dt, double Rm, co
     const unsigned grid = (unsigned)((M + 1 + kStaticBlock - 1) / kStaticBlock);
     unsigned char* sp = (unsigned char*)scratch;
     if (model == PIMC_MODEL_HH)
-        action_static_kernel<HH<double>><<<grid, kStaticBlock, 0, s>>>(M, dt, Rm, rf[0], rf[1], rf[2], rf[3], X_dev,
+        action_static_kernel<HH<double>><<<grid, kStaticBlock, 0, s>>>(hh_fixed_of(dt), M, dt, Rm, rf[0], rf[1], rf[2], rf[3], X_dev,
                                                                       p_dev, y_dev, I_dev, out_dev, sp);
     else if (model == PIMC_MODEL_LINGAUSS)
-        action_static_kernel<LinGauss<double>><<<grid, kStaticBlock, 0, s>>>(M, dt, Rm, rf[0], rf[1], rf[2], rf[3],
+        action_static_kernel<LinGauss<double>><<<grid, kStaticBlock, 0, s>>>(hh_fixed_of(dt), M, dt, Rm, rf[0], rf[1], rf[2], rf[3],
                                                                             X_dev, p_dev, y_dev, I_dev, out_dev, sp);
     else
-        action_static_kernel<Toy1D<double>><<<grid, kStaticBlock, 0, s>>>(M, dt, Rm, rf[0], rf[1], rf[2], rf[3],
+        action_static_kernel<Toy1D<double>><<<grid, kStaticBlock, 0, s>>>(hh_fixed_of(dt), M, dt, Rm, rf[0], rf[1], rf[2], rf[3],
                                                                          X_dev, p_dev, y_dev, I_dev, out_dev, sp);
     if (cudaGetLastError() != cudaSuccess) {
         set_thread_error("pimc_action_static: kernel launch failed");

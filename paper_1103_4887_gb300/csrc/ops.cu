@@ -198,7 +198,7 @@ __global__ void forecast_kernel(Ctx c, int64_t n_steps, const double* I, int n_e
         o[(int64_t)a * (n_steps + 1)] = (double)x[a];
     }
     for (int64_t k = 0; k < n_steps; ++k) {
-        rk4_map<Model, R>(x, q, R(I[k]), R(c.dt), fx);
+        map_step<Model, R>(c.fx, x, q, R(I[k]), R(c.dt), fx);
         if (noise) {
             for (int pair = 0; 2 * pair < D; ++pair) {
                 double z0, z1;
@@ -386,10 +386,10 @@ static cudaError_t map_rate_t(int n_sm, int64_t iters, float* out, cudaStream_t 
     return cudaGetLastError();
 }
 
-// The FP64 form of the same probe: the FP64 HH map (rk4_map<HH<double>>, the
-// map of the plain FP64 sweep) iterated from registers, one state a thread.
+// The FP64 form of the same probe: the FP64 HH map (the map of the plain FP64
+// sweep, in fixed point) iterated from registers, one state a thread.
 template <int MINB>
-__global__ void __launch_bounds__(256, MINB) map_rate_fp64_kernel(int64_t iters, float* out)
+__global__ void __launch_bounds__(256, MINB) map_rate_fp64_kernel(HhFixed fx, int64_t iters, float* out)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     double x[4] = {-65.0 + 0.001 * (double)(t & 1023), 0.05, 0.6, 0.32};
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(256, MINB) map_rate_fp64_kernel(int64_t iters,
     HH<double>::prep(ps, q);
     for (int64_t it = 0; it < iters; ++it) {
         double f[4];
-        rk4_map<HH<double>, double>(x, q, 10.0, 0.02, f);
+        map_step<HH<double>, double>(fx, x, q, 10.0, 0.02, f);
 #pragma unroll
         for (int a = 0; a < 4; ++a) x[a] = f[a];
     }
@@ -408,9 +408,10 @@ __global__ void __launch_bounds__(256, MINB) map_rate_fp64_kernel(int64_t iters,
 cudaError_t launch_map_rate(int packed, int ctas_per_sm, int n_sm, int64_t iters, float* out, cudaStream_t s)
 {
     if (packed == 2) {  // FP64
-        if (ctas_per_sm == 1) map_rate_fp64_kernel<1><<<n_sm, 256, 0, s>>>(iters, out);
-        else if (ctas_per_sm == 2) map_rate_fp64_kernel<2><<<n_sm * 2, 256, 0, s>>>(iters, out);
-        else map_rate_fp64_kernel<4><<<n_sm * 4, 256, 0, s>>>(iters, out);
+        const HhFixed fx = hh_fixed_of(0.02);
+        if (ctas_per_sm == 1) map_rate_fp64_kernel<1><<<n_sm, 256, 0, s>>>(fx, iters, out);
+        else if (ctas_per_sm == 2) map_rate_fp64_kernel<2><<<n_sm * 2, 256, 0, s>>>(fx, iters, out);
+        else map_rate_fp64_kernel<4><<<n_sm * 4, 256, 0, s>>>(fx, iters, out);
         return cudaGetLastError();
     }
     if (packed) {

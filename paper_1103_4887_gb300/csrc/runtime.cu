@@ -134,6 +134,7 @@ Ctx make_ctx(pimc_t h)
     c.chain = h->chain; c.wait_ns = h->wait_ns; c.skip_cta = h->skip_cta;
     c.tile = h->tile;
     c.chk = h->chk;
+    c.fx = hh_fixed_of(h->dt);
     return c;
 }
 

@@ -36,7 +36,7 @@ __device__ __forceinline__ int64_t drive_index(const Ctx& c, int64_t n)
 template <class Model, class R>
 __device__ __forceinline__ void cache_value_at(const Ctx& c, const Coef<R>& k, const R* x, const R* q, R drive, R* g)
 {
-    if (c.scheme == kSchemeRK4) rk4_map<Model, R>(x, q, drive, k.dt, g);
+    if (c.scheme == kSchemeRK4) map_step<Model, R>(c.fx, x, q, drive, k.dt, g);
     else Model::rhs(x, q, drive, g);
 }
 

@@ -276,9 +276,9 @@ __device__ __forceinline__ R site_delta(const Ctx& c, const Coef<R>& k, int64_t 
 
 // Proposal increments of site n at sweep s: D Box-Muller normals (cos then
 // sin per pair of blocks 0, 1) or U(-1, 1) from the same words, and the
-// accept uniform (block 2).
+// E = -log u of the accept uniform u (block 2).
 template <class Model, class R>
-__device__ __forceinline__ void site_draws(const Ctx& c, long long s, int64_t n, R* z, R& u)
+__device__ __forceinline__ void site_draw(const Ctx& c, long long s, int64_t n, R* z, R& E)
 {
     constexpr int D = Model::D;
 #pragma unroll
@@ -295,17 +295,7 @@ __device__ __forceinline__ void site_draws(const Ctx& c, long long s, int64_t n,
         if (2 * pair + 1 < D) z[2 * pair + 1] = z1;
     }
     const uint4 w = draw_block(c.seed, c.chain, (uint64_t)s, (uint32_t)n, kKindSite, 2u);
-    u = Num<R>::uni(w.x, w.y);
-}
-
-// The draws of site n's move at sweep s: the proposal increments z and
-// E = -log u of the accept uniform.
-template <class Model, class R>
-__device__ __forceinline__ void site_draw(const Ctx& c, long long s, int64_t n, R* z, R& E)
-{
-    R u;
-    site_draws<Model, R>(c, s, n, z, u);
-    E = neglog<R>(u);
+    E = neglog_uniform<R>(w.x, w.y);
 }
 
 // The proposal from its increments: x' = x + sigma z (one fma a component)
@@ -404,7 +394,7 @@ __device__ __forceinline__ R param_term(const Ctx& c, const Coef<R>& k, int64_t 
         xn1[a] = X[a * c.ldx + n + 1];
         fc[a] = Fc[a * c.ldf + n];
     }
-    rk4_map<Model, R>(x, pq, ((const R*)c.I)[n], k.dt, fp);
+    map_step<Model, R>(c.fx, x, pq, ((const R*)c.I)[n], k.dt, fp);
 #pragma unroll
     for (int a = 0; a < D; ++a) Fn[a * c.ldf + n] = fp[a];
     if constexpr (std::is_same<R, float>::value) {
@@ -755,7 +745,7 @@ __device__ __forceinline__ void param_draw(const Ctx& c, long long s, int l, dou
     if (c.proposal == kProposalUniform) z = 2.0 * u01d(wz.x, wz.y) - 1.0;
     else Num<double>::box_muller(wz, z, z1);
     const uint4 w = draw_block(c.seed, c.chain, (uint64_t)s, (uint32_t)l, kKindParam, 1u);
-    elog = -log(u01d(w.x, w.y));
+    elog = fx_neglog_uniform(w.x, w.y);
 }
 
 // This sweep's proposal for parameter l (one thread per parameter) from its
@@ -1014,9 +1004,12 @@ __device__ void sweep_chain_general(const Ctx& c, int64_t n0, int64_t n1, int64_
         // tile's flag of the previous sweep (its last site and cache final;
         // the launch orders the first sweep), the last site for the next
         // tile's even flag of this sweep (its first site moved); nothing else
-        // crosses a tile, so a CTA barrier ends each phase.
-#pragma unroll
+        // crosses a tile, so a CTA barrier ends each phase.  FP64: one copy of
+        // the phase's code (the fixed-point map and draws are some 2000
+        // instructions; two copies cost instruction-cache misses).
+#pragma unroll(sizeof(R) == 8 ? 1 : 2)
         for (int parity = 0; parity < 2; ++parity) {
+            unsigned n_acc = 0u, n_prop = 0u;
             R* Fc = (R*)c.F[sh.fidx];
             const int64_t first = n0 + (((n0 & 1) != parity) ? 1 : 0);
             for (int64_t n = first + 2 * (int64_t)tid; n < n1; n += 2 * NT) {
@@ -1038,9 +1031,13 @@ __device__ void sweep_chain_general(const Ctx& c, int64_t n0, int64_t n1, int64_
                         if (!ok) continue;  // leaving: the phase's CTA barrier reads the abort
                     }
                 }
-                my_acc[parity] += site_move<Model, R>(c, kc, n, s, pr, beta, Fc, my_nf) ? 1ull : 0ull;
-                my_prop[parity] += 1ull;
+                n_acc += site_move<Model, R>(c, kc, n, s, pr, beta, Fc, my_nf) ? 1u : 0u;
+                n_prop += 1u;
             }
+            my_acc[0] += parity == 0 ? n_acc : 0u;
+            my_acc[1] += parity == 1 ? n_acc : 0u;
+            my_prop[0] += parity == 0 ? n_prop : 0u;
+            my_prop[1] += parity == 1 ? n_prop : 0u;
             if (Sync::tiled && sync.site_flags) {
                 __syncthreads();
                 if (sh.abort) goto done;
@@ -1143,7 +1140,7 @@ __device__ __forceinline__ void move_values(const Ctx& c, const Coef<R>& k, bool
                                             const R* xn, R drive, R drive1, const R* q, R* f, R* fn)
 {
     if (!trap) {
-        if (has_next) rk4_map<Model, R>(x, q, drive, k.dt, f);
+        if (has_next) map_step<Model, R>(c.fx, x, q, drive, k.dt, f);
     } else {
         Model::rhs(x, q, drive, f);
         if (has_next) Model::rhs(xn, q, drive1, fn);
@@ -1232,8 +1229,7 @@ __device__ void sweep_chain_resident(const Ctx& c, int64_t n0, int64_t n1, int64
         const long long s = sh.sweep;
         const unsigned long long ep = sh.ep0 + (unsigned long long)k + 1ull;
         // this sweep's parameter draws, evaluated before the launch by
-        // param_draws_kernel (FP64 transcendental functions issue slowly on one
-        // warp and would hold up the even phase)
+        // param_draws_kernel (on one warp they would hold up the even phase)
         if (tid < NP && ((sh.free_mask >> tid) & 1u))
             set_param_proposal<Model, R, NT>(sh, tid, __ldg(c.pdraw + 2 * (k * NP + tid)),
                                              __ldg(c.pdraw + 2 * (k * NP + tid) + 1));
@@ -1601,48 +1597,19 @@ __global__ void __launch_bounds__(kSweepBlock, SweepBounds<R>::min_blocks) sweep
 
 // The parameter draws of the next n sweeps of a chain: out[2 (k NP + l)] = z,
 // out[2 (k NP + l) + 1] = -log u for sweep st->sweep + k -- the same values
-// the sweep draws itself (param_draw).  Four lanes a (sweep, parameter) take
-// the three independent FP64 chains in parallel (FP64 issues slowly on this
-// part, so the draws' latency, ahead of every resident launch, is the longest
-// chain): the Box-Muller radius sqrt(-2 log u1), the cosine cos(2 pi u2) and
-// -log u of the accept uniform; z = radius * cosine as in the one-thread form.
-// Also zeroes the three rotating accumulator slots of the exact sums.
+// the sweep draws itself (param_draw); one thread a (sweep, parameter).  Also
+// zeroes the three rotating accumulator slots of the exact sums.
 template <int NP>
-__global__ void __launch_bounds__(256) param_draws_kernel(Ctx c, int64_t n, double* out)
+__global__ void __launch_bounds__(64) param_draws_kernel(Ctx c, int64_t n, double* out)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t < 12) ((unsigned long long*)c.partials)[t] = 0ull;
-    const int64_t idx = t >> 2;  // (sweep, parameter)
-    const int role = (int)(t & 3);
-    const bool valid = idx < n * NP;
-    const int l = (int)(idx % NP);
-    const long long s = c.st->sweep + idx / NP;
-    const bool draw = valid && ((c.st->free_mask >> l) & 1u);
-    double v = 0.0;
-    if (draw) {
-        if (role < 2) {
-            const uint4 wz = draw_block(c.seed, c.chain, (uint64_t)s, (uint32_t)l, kKindParam, 0u);
-            if (c.proposal == kProposalUniform) {
-                v = role == 0 ? 2.0 * u01d(wz.x, wz.y) - 1.0 : 1.0;
-            } else if (role == 0) {
-                v = sqrt(-2.0 * log(u01d(wz.x, wz.y)));
-            } else {
-                double sn, cs;
-                sincospi(2.0 * u01d(wz.z, wz.w), &sn, &cs);
-                v = cs;
-            }
-        } else if (role == 2) {
-            const uint4 w = draw_block(c.seed, c.chain, (uint64_t)s, (uint32_t)l, kKindParam, 1u);
-            v = -log(u01d(w.x, w.y));
-        }
-    }
-    // lanes 4j..4j+3 of a warp hold one (sweep, parameter)
-    const double cosv = __shfl_down_sync(0xffffffffu, v, 1);
-    const double elog = __shfl_down_sync(0xffffffffu, v, 2);
-    if (valid && role == 0) {
-        out[2 * idx] = draw ? (c.proposal == kProposalUniform ? v : v * cosv) : 0.0;
-        out[2 * idx + 1] = draw ? elog : 0.0;
-    }
+    if (t >= n * NP) return;
+    const int l = (int)(t % NP);
+    double z = 0.0, elog = 0.0;
+    if ((c.st->free_mask >> l) & 1u) param_draw(c, c.st->sweep + t / NP, l, z, elog);
+    out[2 * t] = z;
+    out[2 * t + 1] = elog;
 }
 
 // Resident form (FP32-mixed): tiles of at most kSweepBlock - 32 sites, even
@@ -1760,8 +1727,8 @@ static cudaError_t launch_sweep_t(const Ctx& c, int64_t n_sweeps, int grid, int 
     const bool res = resident && resident_fits(prec_of<R>(), c.tile, grid) && c.pdraw && n_sweeps <= kDrawChunk;
     if (res && n_sweeps > 0) {
         // the draws kernel also zeroes the accumulator slots of the exact sums
-        const int64_t nt = 4 * n_sweeps * Model::NP;
-        param_draws_kernel<Model::NP><<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(c, n_sweeps, const_cast<double*>(c.pdraw));
+        const int64_t nt = std::max<int64_t>(n_sweeps * Model::NP, 12);
+        param_draws_kernel<Model::NP><<<(unsigned)((nt + 63) / 64), 64, 0, s>>>(c, n_sweeps, const_cast<double*>(c.pdraw));
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     } else {
