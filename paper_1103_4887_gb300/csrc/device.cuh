@@ -243,6 +243,14 @@ template <class T> struct HHLanes {
     // reaches an addition is an fma result (see the lane rules above).
     static __device__ __forceinline__ void rhs(const T* x, const T* q, T I, T* F, HHCache<T>& k)
     {
+        gates(x, F, k);
+        const T m3h = lmul(lmul(lmul(x[1], x[1]), x[1]), x[2]);
+        const T n2 = lmul(x[3], x[3]);
+        F[0] = current(x[0], m3h, lmul(n2, n2), q, I);
+    }
+    // dm/dt, dh/dt, dn/dt into F[1..3]: independent of the parameters.
+    static __device__ __forceinline__ void gates(const T* x, T* F, HHCache<T>& k)
+    {
         const T V = x[0], m = x[1], h = x[2], n = x[3];
         cache_at(V, k);
         const T um = um_of(V), un = un_of(V);
@@ -258,12 +266,33 @@ template <class T> struct HHLanes {
         F[1] = lfnma(lfma(splat<T>(4.0f), k.e18, a0), m, a0);
         F[2] = lfnma(lfma(lmul(k.dm, k.dn), k.r, a1), h, a1);
         F[3] = lfnma(lfma(splat<T>(0.125f), k.E, a2), n, a2);
+    }
+    // dV/dt from the gate products m^3 h and n^4.
+    static __device__ __forceinline__ T current(T V, T m3h, T n4, const T* q, T I)
+    {
         const T iC = q[7];
-        const T m3h = lmul(lmul(lmul(m, m), m), h);
-        const T n2 = lmul(n, n), n4 = lmul(n2, n2);
         T acc = lfnma(lmul(lmul(q[0], iC), m3h), lsub(V, q[3]), lmul(I, iC));
         acc = lfnma(lmul(lmul(q[1], iC), n4), lsub(V, q[4]), acc);
-        F[0] = lfnma(lmul(q[2], iC), lsub(V, q[5]), acc);
+        return lfnma(lmul(q[2], iC), lsub(V, q[5]), acc);
+    }
+};
+
+// What the first RK4 stage at a state takes that no parameter enters: the gate
+// derivatives and the gate products of the currents.  A site's parameter moves
+// share it (the path stands still during them).
+struct HHStage1 {
+    float k[3], m3h, n4;
+    __device__ __forceinline__ void at(const float* x)
+    {
+        float F[4];
+        HHCache<float> c;
+        HHLanes<float>::gates(x, F, c);
+        k[0] = F[1];
+        k[1] = F[2];
+        k[2] = F[3];
+        m3h = lmul(lmul(lmul(x[1], x[1]), x[1]), x[2]);
+        const float n2 = lmul(x[3], x[3]);
+        n4 = lmul(n2, n2);
     }
 };
 
@@ -271,11 +300,33 @@ template <class T> struct HHLanes {
 // f = x + dt/6 (k1 + 2 k2 + 2 k3 + k4); hdt = dt/2 and sdt = dt/6 as formed
 // by the caller.
 template <class T>
+__device__ __forceinline__ void hh_rk4_rest(const T* x, const T* q, T I, T dt, T hdt, T sdt, T* k, T* f);
+template <class T>
 __device__ __forceinline__ void hh_rk4_lanes(const T* x, const T* q, T I, T dt, T hdt, T sdt, T* f)
 {
-    T k[4], xs[4], acc[4];
+    T k[4];
     HHCache<T> c;
     HHLanes<T>::rhs(x, q, I, k, c);
+    hh_rk4_rest<T>(x, q, I, dt, hdt, sdt, k, f);
+}
+
+// The same from the first stage's parameter-free part (x the same state in
+// every lane): bit for bit the same map.
+template <class T>
+__device__ __forceinline__ void hh_rk4_lanes_from(const HHStage1& s1, const T* x, const T* q, T I, T dt, T hdt, T sdt,
+                                                  T* f)
+{
+    T k[4] = {HHLanes<T>::current(x[0], splat<T>(s1.m3h), splat<T>(s1.n4), q, I), splat<T>(s1.k[0]), splat<T>(s1.k[1]),
+              splat<T>(s1.k[2])};
+    hh_rk4_rest<T>(x, q, I, dt, hdt, sdt, k, f);
+}
+
+// Stages 2 to 4, given k = F(x).
+template <class T>
+__device__ __forceinline__ void hh_rk4_rest(const T* x, const T* q, T I, T dt, T hdt, T sdt, T* k, T* f)
+{
+    T xs[4], acc[4];
+    HHCache<T> c;
 #pragma unroll
     for (int a = 0; a < 4; ++a) { acc[a] = k[a]; xs[a] = lfma(hdt, k[a], x[a]); }
     HHLanes<T>::rhs(xs, q, I, k, c);

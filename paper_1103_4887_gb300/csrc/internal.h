@@ -16,6 +16,7 @@ constexpr int kMaxGrid = 4096;       // upper bound on CTAs of a launch (partial
 constexpr int kMaxSel = 64;          // histogram components
 constexpr int kMaxBins = 4096;
 constexpr int kDrawChunk = 4096;   // sweeps a launch (the parameter-draw buffer's capacity)
+constexpr int kMaxResidentGrid = 511;  // CTAs of a resident launch (the counted sums' fields)
 constexpr int kRedStride = 16;     // per-CTA double slots of the single-pass reductions' scratch
 
 // Scalar sampler state living in device memory.  The sweep kernel keeps a
@@ -49,7 +50,9 @@ struct Ctx {
     void* sig;                    // R[D][ldx]
     uint32_t* acc_win;            // [ldx] accepted moves per site in the adaptation window
     DevState* st;
-    double* partials;             // [3][4] u64 accumulator slots of the exact parameter-move sums
+    double* partials;             // u64: [3][4] Fix3 slots of the exact parameter-move sums, then the counted words
+    int xstride;                  // u64 between the counted words
+    unsigned long long* halo;     // [2][kMaxResidentGrid][8] halo packets of the resident form
     unsigned* bar;                // [0] the grid barrier's word
     unsigned long long* flags;    // [2][kMaxGrid] neighbour epoch flags of the sweep
     uint64_t ep0;                 // epoch of the sweep before this launch's first (flags only grow)
