@@ -413,9 +413,9 @@ PIMC_HD void hh_fixed_rates(const HhFixed& c, int64_t V, int64_t a[3], int64_t l
     l[2] = an + bn;
 }
 
-// Increments dt F of one stage: K[0] of V (format 49), K[1..3] of the gates (format 59).  V (55) and the gates (61) are
+// Increments dt F of one stage: K[0] of V (format 50), K[1..3] of the gates (format 59).  V (55) and the gates (61) are
 // in range on entry; false when a current leaves its format.
-PIMC_HD bool hh_fixed_stage(const HhFixed& c, const HhFixedParams& p, int64_t I47, int64_t V, const int64_t* s,
+PIMC_HD bool hh_fixed_stage(const HhFixed& c, const HhFixedParams& p, int64_t I45, int64_t V, const int64_t* s,
                             int64_t* K)
 {
     int64_t a[3], l[3];
@@ -424,21 +424,23 @@ PIMC_HD bool hh_fixed_stage(const HhFixed& c, const HhFixedParams& p, int64_t I4
     for (int g = 0; g < 3; ++g) K[1 + g] = (a[g] >> 1) - fx_smul(l[g] * 4, s[g]);
     const int64_t m = s[0] * 2, h = s[1] * 2, n = s[2] * 2;  // format 62
     const int64_t m2 = fx_smul(m, m) * 4, mh = fx_smul(m, h) * 4, n2 = fx_smul(n, n) * 4;
-    const int64_t m3h = fx_smul(m2, mh) * 4, n4 = fx_smul(n2, n2) * 4;
-    const int64_t tNa = fx_smul(V - p.ENa, m3h), tK = fx_smul(V - p.EK, n4);  // format 53
-    constexpr int64_t kNa = 1ll << 59, kK4 = 1ll << 61;                      // 64, 256
-    const bool ok = fx_inside(tNa, kNa) && fx_inside(tK, kK4);
-    const int64_t S = I47 - fx_smul(p.gNa, (int64_t)((uint64_t)tNa << 3)) - fx_smul(p.gK, (int64_t)((uint64_t)tK << 1)) -
-                      (fx_smul(p.gL, V - p.EL) >> 4);
-    K[0] = fx_smul(S, p.kappa);
-    constexpr int64_t kK = 100ll << 49;
-    return ok && fx_inside(K[0], kK);
+    const int64_t m3h = fx_smul(m2, mh), n4 = fx_smul(n2, n2);                // format 60
+    const int64_t tNa = fx_smul(V - p.ENa, (int64_t)((uint64_t)m3h << 2));    // format 53
+    const int64_t tK = fx_smul(V - p.EK, (int64_t)((uint64_t)n4 << 2));
+    constexpr int64_t kTwo = 1ll << 61, kT = 1ll << 61, kS = 1ll << 59;       // 2, 256, 2^14
+    const bool ok = fx_inside(m3h, kTwo) && fx_inside(n4, kTwo) && fx_inside(tNa, kT) && fx_inside(tK, kT);
+    const int64_t S = I45 - fx_smul(p.gNa, (int64_t)((uint64_t)tNa << 1)) -
+                      (fx_smul(p.gK, (int64_t)((uint64_t)tK << 1)) >> 2) - (fx_smul(p.gL, V - p.EL) >> 6);
+    K[0] = fx_smul((int64_t)((uint64_t)S << 3), p.kappa);
+    constexpr int64_t kK = 100ll << 50;
+    return ok && fx_inside(S, kS) && fx_inside(K[0], kK);
 }
 
-// Whether a state in fixed point is inside the range of the stage: |V| < 100, |gate| < 1.18.
+// Whether a state in fixed point is inside the range of the stage: |V| < 100, |gate| < 1.41 (their products of two stay
+// below 2; sampled gates scatter past 1 at the spikes).
 PIMC_HD bool hh_fixed_inside(int64_t V, const int64_t* s)
 {
-    constexpr int64_t kV = 100ll << 55, kS = 0x25c28f5c00000000ll;  // 1.18, format 61
+    constexpr int64_t kV = 100ll << 55, kS = 0x2d1eb85100000000ll;  // 1.41, format 61
     return fx_inside(V, kV) && fx_inside(s[0], kS) && fx_inside(s[1], kS) && fx_inside(s[2], kS);
 }
 
@@ -446,21 +448,21 @@ PIMC_HD bool hh_fixed_inside(int64_t V, const int64_t* s)
 // leaves the range of the formats.
 PIMC_HD bool hh_map_fixed(const HhFixed& c, const HhFixedParams& p, const double* x, double I, double* f)
 {
-    if (!p.ok || !fx_below(x[0], 100.0) || !fx_below(x[1], 1.125) || !fx_below(x[2], 1.125) ||
-        !fx_below(x[3], 1.125) || !fx_below(I, 16384.0))
+    if (!p.ok || !fx_below(x[0], 100.0) || !fx_below(x[1], 1.375) || !fx_below(x[2], 1.375) ||
+        !fx_below(x[3], 1.375) || !fx_below(I, 16384.0))
         return false;
-    const int64_t V0 = fx_of(x[0], 55), I47 = fx_of(I, 47);
+    const int64_t V0 = fx_of(x[0], 55), I45 = fx_of(I, 45);
     int64_t s0[3], V = V0, s[3], aV = 0, as[3] = {0, 0, 0}, K[4];
     for (int g = 0; g < 3; ++g) s[g] = s0[g] = fx_of(x[1 + g], 61);
     bool ok = true;
     // one copy of the stage's code: four would not fit the instruction cache
 #pragma unroll 1
     for (int st = 0; st < 4; ++st) {
-        ok = hh_fixed_stage(c, p, I47, V, s, K);
+        ok = hh_fixed_stage(c, p, I45, V, s, K);
         if (!ok) return false;
         const int w = (st == 1 || st == 2) ? 1 : 0, d = st < 2 ? 0 : 1;  // weight 2^w; next stage at x + K 2^(d - 1)
         aV += K[0] << w;
-        V = V0 + (K[0] << (5 + d));
+        V = V0 + (K[0] << (4 + d));
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
             as[g] += K[1 + g] << w;
@@ -469,7 +471,7 @@ PIMC_HD bool hh_map_fixed(const HhFixed& c, const HhFixedParams& p, const double
         if (st < 3 && !hh_fixed_inside(V, s)) return false;
     }
     constexpr int64_t kSixth = 0x5555555555555555ll;  // 1/6, format 65
-    f[0] = fx_double(V0 + fx_smul(aV * 16, kSixth) * 2, 55);
+    f[0] = fx_double(V0 + fx_smul(aV * 8, kSixth) * 2, 55);
 #pragma unroll
     for (int g = 0; g < 3; ++g) f[1 + g] = fx_double(s0[g] + fx_smul(as[g], kSixth) * 2, 61);
     return true;
