@@ -155,7 +155,10 @@ cudaError_t launch_convert(int prec, const double* src, void* dst, int64_t n, cu
 // Ensemble forecast from the current state: out[e][a][k] (device, FP64).
 cudaError_t launch_forecast(int model, int prec, const Ctx& c, int64_t n_steps, const double* I, int n_ens,
                             int noise, uint64_t seed, double* out, cudaStream_t s);
-// X conversion between the handle storage and dense FP64 [D][M+1].
-cudaError_t launch_path_io(int prec, const Ctx& c, int D, double* dense, int to_state, cudaStream_t s);
+// rows x n values of a storage array (row stride ld) to dense FP64 rows.
+cudaError_t launch_rows_out(int prec, const void* src, int64_t ld, int rows, int64_t n, double* dense, cudaStream_t s);
+// Moments from the running sums (shift may be null): mean or var (the other null) of n quantities.
+cudaError_t launch_moments(const double* S1, const double* S2, const double* shift, int64_t n, double J, double* mean,
+                           double* var, cudaStream_t s);
 
 }  // namespace pimc

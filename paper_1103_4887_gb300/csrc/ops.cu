@@ -229,17 +229,26 @@ __global__ void convert_kernel(const double* src, R* dst, int64_t n)
     if (i < n) dst[i] = R(src[i]);
 }
 
-// Handle storage <-> dense FP64 [D][M+1].
+// Rows of the handle's storage type ([gridDim.y][ld], n columns each) to dense
+// FP64 rows.
 template <class R>
-__global__ void path_io_kernel(Ctx c, int D, double* dense, int to_state)
+__global__ void rows_out_kernel(const R* src, int64_t ld, int64_t n, double* dense)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t tot = (int64_t)D * (c.M + 1);
-    if (i >= tot) return;
-    const int64_t a = i / (c.M + 1), n = i - a * (c.M + 1);
-    R* X = (R*)c.X;
-    if (to_state) X[a * c.ldx + n] = R(dense[i]);
-    else dense[i] = (double)X[a * c.ldx + n];
+    if (i < n) dense[blockIdx.y * n + i] = (double)src[blockIdx.y * ld + i];
+}
+
+// mean = shift + S1/J or var = (S2 - S1^2/J)/(J - 1) of n quantities (one of the
+// outputs null; shift may be null), NaN where J is too small.  The same operations in the same order
+// as the formula on the host: no multiply-add is fused.
+__global__ void moments_kernel(const double* S1, const double* S2, const double* shift, int64_t n, double J, double* mean,
+                               double* var)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double s1 = S1[i], m = __ddiv_rn(s1, J), nan = __longlong_as_double(0x7ff8000000000000ll);
+    if (mean) mean[i] = J > 0.0 ? (shift ? __dadd_rn(shift[i], m) : m) : nan;
+    else var[i] = J > 1.0 ? __ddiv_rn(__dsub_rn(S2[i], __ddiv_rn(__dmul_rn(s1, s1), J)), __dsub_rn(J, 1.0)) : nan;
 }
 
 // ---------------------------------------------------------------------------
@@ -326,12 +335,18 @@ cudaError_t launch_convert(int prec, const double* src, void* dst, int64_t n, cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_path_io(int prec, const Ctx& c, int D, double* dense, int to_state, cudaStream_t s)
+cudaError_t launch_rows_out(int prec, const void* src, int64_t ld, int rows, int64_t n, double* dense, cudaStream_t s)
 {
-    const int64_t tot = (int64_t)D * (c.M + 1);
-    const unsigned grid = (unsigned)((tot + 255) / 256);
-    if (prec == 0) path_io_kernel<double><<<grid, 256, 0, s>>>(c, D, dense, to_state);
-    else path_io_kernel<float><<<grid, 256, 0, s>>>(c, D, dense, to_state);
+    const dim3 grid((unsigned)((n + 255) / 256), (unsigned)rows);
+    if (prec == 0) rows_out_kernel<double><<<grid, 256, 0, s>>>((const double*)src, ld, n, dense);
+    else rows_out_kernel<float><<<grid, 256, 0, s>>>((const float*)src, ld, n, dense);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_moments(const double* S1, const double* S2, const double* shift, int64_t n, double J, double* mean,
+                           double* var, cudaStream_t s)
+{
+    moments_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(S1, S2, shift, n, J, mean, var);
     return cudaGetLastError();
 }
 
