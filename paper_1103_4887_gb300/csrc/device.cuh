@@ -186,6 +186,13 @@ __device__ __forceinline__ float2 lsel_small(float2 u, float cut, float2 s, floa
     return make_float2(lsel_small(u.x, cut, s.x, v.x), lsel_small(u.y, cut, s.y, v.y));
 }
 
+// Whether |u| or |v| is below cut in any lane
+__device__ __forceinline__ bool lany_small(float u, float v, float cut) { return fminf(fabsf(u), fabsf(v)) < cut; }
+__device__ __forceinline__ bool lany_small(float2 u, float2 v, float cut)
+{
+    return fminf(fminf(fabsf(u.x), fabsf(u.y)), fminf(fabsf(v.x), fabsf(v.y))) < cut;
+}
+
 // The transcendental part of the HH rates at V (see HH below): E = e^{-(V+65)/80},
 // e^{-(V+65)/18}, the psi denominators dm, dn and the reciprocal r = 1/(dm dn dh).
 template <class T> struct HHCache {
@@ -252,11 +259,28 @@ template <class T> struct HHLanes {
     static __device__ __forceinline__ void gates(const T* x, T* F, HHCache<T>& k)
     {
         const T V = x[0], m = x[1], h = x[2], n = x[3];
-        cache_at(V, k);
+        // cache_at and the psi numerators.  Packed lanes keep the series behind a
+        // branch that few warps take (two windows of 0.2 mV): fewer instructions
+        // than selects on every lane, the same bits.  Single lanes, which run
+        // where latency counts, select (HMC trajectory 139 us, 144 with the
+        // branch).
+        const T t = ladd(V, splat<T>(65.0f));
+        k.E = lex2(lmul(t, splat<T>(float(-kLog2e / 80.0))));
+        k.e18 = lex2(lmul(t, splat<T>(float(-kLog2e / 18.0))));
         const T um = um_of(V), un = un_of(V);
-        const T nm = lsel_small(um, kCut, psi_series(um), um);
-        const T nn = lsel_small(un, kCut, psi_series(un), un);
+        const T one = splat<T>(1.0f);
+        k.dm = lsub(one, lex2(lmul(um, splat<T>(float(-kLog2e)))));
+        k.dn = lsub(one, lex2(lmul(un, splat<T>(float(-kLog2e)))));
+        T nm = um, nn = un;
+        constexpr bool kPacked = std::is_same<T, float2>::value;
+        if (!kPacked || __builtin_expect(lany_small(um, un, kCut), 0)) {
+            nm = lsel_small(um, kCut, psi_series(um), um);
+            nn = lsel_small(un, kCut, psi_series(un), un);
+            k.dm = lsel_small(um, kCut, one, k.dm);
+            k.dn = lsel_small(un, kCut, one, k.dn);
+        }
         const T dh = dh_of(k.E);
+        k.r = lrcp(lmul(lmul(k.dm, k.dn), dh));
         const T E2 = lmul(k.E, k.E), E4 = lmul(E2, E2);
         const T a0 = lmul(nm, lmul(lmul(k.dn, dh), k.r));
         const T a1 = lmul(splat<T>(0.07f), E4);

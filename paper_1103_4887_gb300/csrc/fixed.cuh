@@ -136,6 +136,18 @@ PIMC_HD double fx_from_bits(uint64_t b)
 #endif
 }
 
+// The double equal to v: normal values by integer operations (the conversion instruction queues for the FP64 pipe).
+PIMC_HD double fx_widen(float v)
+{
+#ifdef __CUDA_ARCH__
+    const uint32_t b = __float_as_uint(v), e = b & 0x7f800000u;
+    if (__builtin_expect(e == 0u || e == 0x7f800000u, 0)) return (double)v;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+#else
+    return (double)v;
+#endif
+}
+
 // |v| < lim for a lim whose low word is zero (false for NaN): a comparison of high words.
 PIMC_HD bool fx_below(double v, double lim)
 {

@@ -28,6 +28,9 @@ __device__ __forceinline__ void accumulate(const Ctx& c, int64_t ci, double v, b
     c.S2[ci] += d * d;
 }
 
+__device__ __forceinline__ double widen(float v) { return fx_widen(v); }
+__device__ __forceinline__ double widen(double v) { return v; }
+
 // Thread t of nt records its share; p is the current parameter vector and Fc
 // the current cache (f(x_n) or F(x_n)), which gives the model-error residuals
 // eps_{n+1} without another map evaluation; the
@@ -49,22 +52,22 @@ __device__ void record_sample(const Ctx& c, int64_t n0, int64_t n1, bool params_
 #pragma unroll
         for (int a = 0; a < D; ++a) {
             const int64_t ci = (int64_t)a * (M + 1) + n;
-            xv[a] = (double)X[a * c.ldx + n];
+            xv[a] = widen(X[a * c.ldx + n]);
             sv[a] = first_rec ? xv[a] : c.shift[ci];
             s1[a] = c.S1[ci];
             s2[a] = c.S2[ci];
             e[a] = r1[a] = r2[a] = 0.0;
             if (has_eps) {
-                const double xn1 = (double)X[a * c.ldx + n + 1];
-                const double gn = (double)Fc[a * c.ldf + n];
-                e[a] = trap ? xn1 - xv[a] - 0.5 * c.dt * ((double)Fc[a * c.ldf + n + 1] + gn) : xn1 - gn;
+                const double xn1 = widen(X[a * c.ldx + n + 1]);
+                const double gn = widen(Fc[a * c.ldf + n]);
+                e[a] = trap ? xn1 - xv[a] - 0.5 * c.dt * (widen(Fc[a * c.ldf + n + 1]) + gn) : xn1 - gn;
                 r1[a] = c.R1[(int64_t)a * M + n];
                 r2[a] = c.R2[(int64_t)a * M + n];
             }
         }
         e[D] = r1[D] = r2[D] = 0.0;
         if (has_d) {
-            e[D] = xv[0] - (double)((const R*)c.y)[n];
+            e[D] = xv[0] - widen(((const R*)c.y)[n]);
             r1[D] = c.R1[(int64_t)D * M + n - 1];
             r2[D] = c.R2[(int64_t)D * M + n - 1];
         }

@@ -565,47 +565,48 @@ __device__ __forceinline__ bool fix_less(Fix3 s, double e)
 }
 
 // A thread's running exact sum of FP32 terms, for loops over many sites: the
-// same integer T = t 2^64 truncated toward zero as fix_add, kept as one
-// 128-bit two's complement integer (hi:lo) -- a shift and a 128-bit add or
-// subtract a term instead of a split into three chunks.  Terms of magnitude
-// 2^36 or more, and non-finite ones, go to the Fix3 sum instead, so up to 2^26
-// terms cannot overflow; acc_fold adds the 128-bit sum into the Fix3 sum.  The
-// total is the same integer either way, so every form keeps the same bits.
-struct Acc128 {
-    unsigned long long lo, hi;
+// same integer T = t 2^64 truncated toward zero as fix_add, kept in three
+// signed 64-bit bins of weight 2^0, 2^32 and 2^64 -- a term's mantissa, shifted
+// by up to 31 bits, is one 32 x 32 + 64 multiply-add into its bin.  A term is
+// below 2^55 in its bin's units, so 255 terms cannot overflow; bins_fold, due
+// at least that often, adds the bins into the Fix3 sum.  Terms outside
+// [2^-40, 2^32) in magnitude go to the Fix3 sum at once.  The total is the same
+// integer either way, so every form keeps the same bits.  16 instructions a
+// term; the 128-bit shift and add it replaces took 30.
+struct Bins {
+    long long b[3];
 };
+constexpr int kBinTerms = 254;
 
-__device__ __forceinline__ void acc_add(Acc128& a, Fix3& big, float t)
+__device__ __forceinline__ void bins_zero(Bins& a) { a.b[0] = a.b[1] = a.b[2] = 0; }
+
+__device__ __forceinline__ void bins_add(Bins& a, Fix3& big, float t)
 {
     const unsigned b = __float_as_uint(t);
-    const unsigned ex = (b >> 23) & 0xffu;
-    if (ex >= 127u + 36u) {
+    const unsigned sh = ((b >> 23) & 0xffu) - 86u;  // bit of T that the mantissa's bit 0 lands on
+    if (sh > 72u) {
         fix_add(big, t);
         return;
     }
-    const unsigned long long man = ex ? (unsigned long long)((b & 0x7fffffu) | 0x800000u) : (unsigned long long)(b & 0x7fffffu);
-    const int sh = (ex ? (int)ex - 150 : -149) + 64;  // bit of T that man's bit 0 lands on (<= 77)
-    unsigned long long lo = 0ull, hi = 0ull;
-    if (sh >= 64) hi = man << (sh - 64);
-    else if (sh > 40) { lo = man << sh; hi = man >> (64 - sh); }
-    else if (sh >= 0) lo = man << sh;
-    else if (sh > -24) lo = man >> (-sh);
-    if (b >> 31) {
-        const unsigned long long l2 = a.lo - lo;
-        a.hi = a.hi - hi - (a.lo < lo ? 1ull : 0ull);
-        a.lo = l2;
-    } else {
-        const unsigned long long l2 = a.lo + lo;
-        a.hi = a.hi + hi + (l2 < lo ? 1ull : 0ull);
-        a.lo = l2;
-    }
+    int man = (int)((b & 0x7fffffu) | 0x800000u);
+    if ((int)b < 0) man = -man;
+    const int pw = 1 << (sh & 31u);
+    const unsigned w = sh >> 5;
+    // 2^31 as a signed factor is negative: its product enters with the sign turned
+    const int f = (sh & 31u) == 31u ? -man : man;
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+        if (w == (unsigned)j) a.b[j] += (long long)f * (long long)pw;
 }
 
-__device__ __forceinline__ void acc_fold(const Acc128& a, Fix3& f)
+// Adds the bins into f (chunk by chunk: c0 + c1 2^42 + c2 2^84) and clears them.
+__device__ __forceinline__ void bins_fold(Bins& a, Fix3& f)
 {
-    f.c[0] += (long long)(a.lo & (unsigned long long)kFixMask);
-    f.c[1] += (long long)(((a.lo >> 42) | (a.hi << 22)) & (unsigned long long)kFixMask);
-    f.c[2] += (long long)a.hi >> 20;
+    // b0 = low 42 bits + rest 2^42; b1 2^32 = (low 10 bits) 2^32 + rest 2^42; b2 2^64 = (low 20 bits) 2^64 + rest 2^84
+    f.c[0] += (a.b[0] & kFixMask) + ((a.b[1] & 0x3ffll) << 32);
+    f.c[1] += (a.b[0] >> 42) + (a.b[1] >> 10) + ((a.b[2] & 0xfffffll) << 22);
+    f.c[2] += a.b[2] >> 20;
+    bins_zero(a);
 }
 
 // Warp sum of Fix3 values, valid in every lane.  Each lane's value is
@@ -1089,7 +1090,9 @@ __device__ __forceinline__ void param_terms_paired(const Ctx& c, const Coef<floa
     for (int j = 0; j < kMaxP; ++j) q2[j] = splat<float2>(pq[j]);
     const float2 dt2 = splat<float2>(k.dt), beta2 = splat<float2>(beta);
     const float2 hdt2 = splat<float2>(__fmul_rn(0.5f, k.dt)), sdt2 = splat<float2>(__fdiv_rn(k.dt, 6.0f));
-    Acc128 acc{0ull, 0ull};
+    Bins acc;
+    bins_zero(acc);
+    int terms = 0;
     PairStage<NT>* st = (PairStage<NT>*)pimc_dyn_smem;
     int64_t n = n0 + 2 * (int64_t)tid;
     // the copies of pair (m, m + 1) into buffer b (m < nend)
@@ -1126,11 +1129,16 @@ __device__ __forceinline__ void param_terms_paired(const Ctx& c, const Coef<floa
             }
         }
         const float2 t = rk4_term_lanes<float2, 4>(beta2, k.Rf, xn1, fp, fc);
-        acc_add(acc, part, t.x);
-        if (two) acc_add(acc, part, t.y);
+        bins_add(acc, part, t.x);
+        if (two) bins_add(acc, part, t.y);
+        terms += 2;
+        if (terms == kBinTerms) {
+            bins_fold(acc, part);
+            terms = 0;
+        }
     }
     cp_async_wait<0>();
-    acc_fold(acc, part);
+    bins_fold(acc, part);
 }
 
 // ---- general form -----------------------------------------------------------
@@ -1479,21 +1487,21 @@ __device__ __forceinline__ void record_site(const Ctx& c, int64_t n, bool first_
 #pragma unroll
     for (int a = 0; a < D; ++a) {
         const int64_t ci = (int64_t)a * (M + 1) + n;
-        xv[a] = (double)x[a];
+        xv[a] = widen(x[a]);
         sv[a] = first_rec ? xv[a] : c.shift[ci];
         s1[a] = c.S1[ci];
         s2[a] = c.S2[ci];
         e[a] = r1[a] = r2[a] = 0.0;
         if (has_eps) {
-            const double x1 = (double)xn1[a], g0 = (double)g[a];
-            e[a] = kTrap ? x1 - xv[a] - 0.5 * c.dt * ((double)gn1[a] + g0) : x1 - g0;
+            const double x1 = widen(xn1[a]), g0 = widen(g[a]);
+            e[a] = kTrap ? x1 - xv[a] - 0.5 * c.dt * (widen(gn1[a]) + g0) : x1 - g0;
             r1[a] = c.R1[(int64_t)a * M + n];
             r2[a] = c.R2[(int64_t)a * M + n];
         }
     }
     e[D] = r1[D] = r2[D] = 0.0;
     if (has_d) {
-        e[D] = xv[0] - (double)yv;
+        e[D] = xv[0] - widen(yv);
         r1[D] = c.R1[(int64_t)D * M + n - 1];
         r2[D] = c.R2[(int64_t)D * M + n - 1];
     }
@@ -2291,18 +2299,26 @@ __global__ void __launch_bounds__(kBlock) param_delta_kernel(Ctx c, int l, doubl
 }
 
 // The exact sum of n terms by one CTA (the test hook of the Fix3 arithmetic;
-// acc128: FP32 terms through the per-thread 128-bit accumulator, as the
-// general form's parameter moves add them).
-template <class T, bool acc128>
+// bins: FP32 terms through the per-thread bins, as the general form's parameter
+// moves add them).
+template <class T, bool bins>
 __global__ void __launch_bounds__(256) fix_sum_kernel(const double* t, int64_t n, double* out)
 {
     __shared__ Fix3 wfix[256 / 32];
     Fix3 f;
     fix_zero(f);
-    if constexpr (acc128) {
-        Acc128 a{0ull, 0ull};
-        for (int64_t i = threadIdx.x; i < n; i += 256) acc_add(a, f, (float)t[i]);
-        acc_fold(a, f);
+    if constexpr (bins) {
+        Bins a;
+        bins_zero(a);
+        int terms = 0;
+        for (int64_t i = threadIdx.x; i < n; i += 256) {
+            bins_add(a, f, (float)t[i]);
+            if (++terms == kBinTerms) {
+                bins_fold(a, f);
+                terms = 0;
+            }
+        }
+        bins_fold(a, f);
     } else {
         for (int64_t i = threadIdx.x; i < n; i += 256) fix_add(f, (T)t[i]);
     }
