@@ -12,12 +12,13 @@
 //
 // Measured: the FP64 map is some 650 FP64 instructions, 49 000 scheduler cycles a warp; this one 5 200 with four warps a
 // scheduler and 9 000 alone (integer ALU and multiply-add pipes together; latency alone).  FP64 sweeps: M = 1000, 3 free
-// parameters, 120 -> 48 us; M = 32768, 7 free, 341 -> 110 us.  Normals by the FP64 functions: some 90 FP64 instructions
+// parameters, 120 -> 48 us; M = 32768, 7 free, 341 -> 94 us.  Normals by the FP64 functions: some 90 FP64 instructions
 // each; here 350 cycles.
 //
 // Integer arithmetic gives the same bits in every kernel and on the host, so the file also compiles as plain C++.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -44,23 +45,34 @@ PIMC_HD uint64_t fx_umul(uint64_t a, uint64_t b)
 }
 
 // a b / 2^64 for signed operands, at most 3 below it: three 32x32 + 64 multiply-adds; the low halves enter with 31
-// bits so that every partial product is a signed one, and their own product is left out.
-// On the device as PTX: compiled from the C++ below it takes 25 cycles a warp instead of 16.
-PIMC_HD int64_t fx_smul(int64_t a, int64_t b)
+// bits so that every partial product is a signed one, and their own product is left out.  kCentred adds what that leaves
+// out on average, 1.25 (sums over a path would collect it); it takes a constant's registers, so only the products that
+// carry a result's last bits use it.  On the device as PTX: compiled from the C++ below it takes 25 cycles a warp
+// instead of 16.
+template <bool kCentred = false> PIMC_HD int64_t fx_smul(int64_t a, int64_t b)
 {
 #ifdef __CUDA_ARCH__
     int64_t r;
-    asm("{\n\t.reg .s32 a0, a1, b0, b1;\n\t.reg .s64 t;\n\t"
-        "mov.b64 {a0, a1}, %1;\n\tmov.b64 {b0, b1}, %2;\n\tshr.u32 a0, a0, 1;\n\tshr.u32 b0, b0, 1;\n\t"
-        "mul.wide.s32 t, a1, b0;\n\tmad.wide.s32 t, a0, b1, t;\n\tshr.s64 t, t, 31;\n\t"
-        "mad.wide.s32 %0, a1, b1, t;\n\t}"
-        : "=l"(r)
-        : "l"(a), "l"(b));
+    if (kCentred) {
+        asm("{\n\t.reg .s32 a0, a1, b0, b1;\n\t.reg .s64 t;\n\t"
+            "mov.b64 {a0, a1}, %1;\n\tmov.b64 {b0, b1}, %2;\n\tshr.u32 a0, a0, 1;\n\tshr.u32 b0, b0, 1;\n\t"
+            "mad.wide.s32 t, a1, b0, 2684354560;\n\tmad.wide.s32 t, a0, b1, t;\n\tshr.s64 t, t, 31;\n\t"
+            "mad.wide.s32 %0, a1, b1, t;\n\t}"
+            : "=l"(r)
+            : "l"(a), "l"(b));
+    } else {
+        asm("{\n\t.reg .s32 a0, a1, b0, b1;\n\t.reg .s64 t;\n\t"
+            "mov.b64 {a0, a1}, %1;\n\tmov.b64 {b0, b1}, %2;\n\tshr.u32 a0, a0, 1;\n\tshr.u32 b0, b0, 1;\n\t"
+            "mul.wide.s32 t, a1, b0;\n\tmad.wide.s32 t, a0, b1, t;\n\tshr.s64 t, t, 31;\n\t"
+            "mad.wide.s32 %0, a1, b1, t;\n\t}"
+            : "=l"(r)
+            : "l"(a), "l"(b));
+    }
     return r;
 #else
     const int32_t a1 = (int32_t)(a >> 32), b1 = (int32_t)(b >> 32);
     const int32_t a0 = (int32_t)((uint32_t)a >> 1), b0 = (int32_t)((uint32_t)b >> 1);
-    const int64_t t = (int64_t)a1 * b0 + (int64_t)a0 * b1;
+    const int64_t t = (int64_t)a1 * b0 + (int64_t)a0 * b1 + (kCentred ? 2684354560ll : 0ll);  // 1.25 2^31
     return (int64_t)a1 * b1 + (t >> 31);
 #endif
 }
@@ -373,11 +385,36 @@ PIMC_HD int64_t fx_psi_series(int64_t v)
     return kFxOne62 + (u >> 4) + fx_smul(fx_smul(u2, 0x555555555555555ll), s3);
 }
 
+// psi'(u) for |u| < 1/16 in format 62: 1/2 + u/6 (1 - u^2/30 (1 - u^2/28 (1 - u^2/30))).
+PIMC_HD int64_t fx_dpsi_series(int64_t v)
+{
+    const int64_t u = fx_smul(v * 256, 0x6666666666666666ll);  // format 65
+    const int64_t u2 = fx_smul(u, u);                          // format 66
+    const int64_t s1 = kFxOne62 - (fx_smul(u2, 0x222222222222222ll) >> 2);
+    const int64_t s2 = kFxOne62 - fx_smul(fx_smul(u2, 0x249249249249249ll), s1);
+    const int64_t s3 = kFxOne62 - fx_smul(fx_smul(u2, 0x222222222222222ll), s2);
+    return (kFxOne62 >> 1) + (fx_smul(fx_smul(u, s3), 0xaaaaaaaaaaaaaabll) * 2);  // u s3: format 63; /6 (1/6, 62): 61
+}
+
+// psi'(u) for |u| >= 1/16 in format 62, from v = 10 u (55), p = 10 psi (52), x and s with 1/|1 - e^{-u}| = x 2^s.
+PIMC_HD int64_t fx_dpsi(int64_t v, int64_t p, int64_t x, int s)
+{
+    const int64_t u = fx_smul(v, 0x6666666666666666ll);                              // format 57
+    const int64_t psi = fx_smul((int64_t)((uint64_t)p << 3), 0x6666666666666666ll);  // format 57
+    int64_t n = ((int64_t)1 << 57) + u - psi;  // the sign of 1 - e^{-u}
+    n = n < 0 ? -n : n;
+    const int64_t q = fx_smul((int64_t)fx_shl((uint64_t)n << 3, s > 0 ? s & 15 : 0), x);  // format 57
+    return fx_sar(q, s < 0 ? -s & 31 : 0) * 32;
+}
+
 // Gate rates at V (format 55, |V| < 100): a[g] = dt alpha, l[g] = dt (alpha + beta) of m, h, n in format 60.  With
 // t = V + 101 in (1, 201): e^{-t/80} and e^{-t/18} from the table, e^{-t/20} and B = e^{-t/10} by squaring mantissas;
 // 1 - e^{-u} of alpha_m and alpha_n and 1 + e^{-(V+35)/10} of beta_h from B scaled by 2^-k, which keeps all three
 // below 1 at every V.
-PIMC_HD void hh_fixed_rates(const HhFixed& c, int64_t V, int64_t a[3], int64_t l[3])
+// With kAdj also d[g] = dt d(alpha)/dV and e[g] = dt d(beta)/dV (format 60):
+// alpha' from psi'(u) = (1 + u - psi)/(1 - e^{-u}), or its series.
+template <bool kAdj>
+PIMC_HD void hh_fixed_rates(const HhFixed& c, int64_t V, int64_t a[3], int64_t l[3], int64_t* da, int64_t* db)
 {
     const uint64_t U = ((uint64_t)V + (101ull << 55)) << 1;                   // t, format 56
     const uint64_t z80 = 0ull - fx_umul(U, 0x93bb62877cdff3c9ull);           // -t log2(e)/80, format 61, modulo 8
@@ -407,16 +444,28 @@ PIMC_HD void hh_fixed_rates(const HhFixed& c, int64_t V, int64_t a[3], int64_t l
     // V + V0), a right shift after it.  u and 1 - e^{-u} have the same sign.
     const int64_t vm = V + (40ll << 55), vn = V + (55ll << 55);
     const int sm = zm - 2 - k, sn = zn - 2 - k, shh = k + 2 - zh;
-    const int64_t pm = fx_sar(fx_smul((int64_t)fx_shl((uint64_t)(vm < 0 ? -vm : vm), sm > 0 ? sm & 15 : 0), xm),
+    const int64_t pm = fx_sar(fx_smul<true>((int64_t)fx_shl((uint64_t)(vm < 0 ? -vm : vm), sm > 0 ? sm & 15 : 0), xm),
                               sm < 0 ? -sm & 31 : 0);
-    const int64_t pn = fx_sar(fx_smul((int64_t)fx_shl((uint64_t)(vn < 0 ? -vn : vn), sn > 0 ? sn & 15 : 0), xn),
+    const int64_t pn = fx_sar(fx_smul<true>((int64_t)fx_shl((uint64_t)(vn < 0 ? -vn : vn), sn > 0 ? sn & 15 : 0), xn),
                               sn < 0 ? -sn & 31 : 0);
-    int64_t am = fx_smul(pm, c.dt10) << 2, an = fx_smul(pn, c.dt100) >> 1;
+    int64_t am = fx_smul<true>(pm, c.dt10) << 2, an = fx_smul<true>(pn, c.dt100) >> 1;
     const int64_t bh = fx_sar(fx_smul(c.dt67, xh), 4 + shh);
     // |u| < 1/16: the series (the quotient above is not used there)
     constexpr int64_t kCut = 5ll << 52;  // 10/16, format 55
-    if (fx_inside(vm, kCut)) am = fx_smul(c.dt67, fx_psi_series(vm)) >> 5;
-    if (fx_inside(vn, kCut)) an = fx_smul(c.dt10, fx_psi_series(vn)) >> 8;
+    const bool cut_m = fx_inside(vm, kCut), cut_n = fx_inside(vn, kCut);
+    if (cut_m) am = fx_smul(c.dt67, fx_psi_series(vm)) >> 5;
+    if (cut_n) an = fx_smul(c.dt10, fx_psi_series(vn)) >> 8;
+    if (kAdj) {
+        const int64_t dm = cut_m ? fx_dpsi_series(vm) : fx_dpsi(vm, pm, xm, sm);
+        const int64_t dn = cut_n ? fx_dpsi_series(vn) : fx_dpsi(vn, pn, xn, sn);
+        da[0] = fx_smul(c.dt10, dm) >> 8;
+        da[1] = fx_smul(ah, -0x666666666666666ll) * 2;                         // -alpha_h/20 (-0.1 in format 62, halved)
+        da[2] = fx_smul(c.dt100, dn) >> 11;
+        db[0] = -fx_smul(bm * 4, 0x38e38e38e38e38ell);                         // -beta_m/18 (1/18 in format 62)
+        const int64_t b61 = fx_sar(xh, shh);                                   // beta_h, format 61
+        db[1] = fx_smul(fx_smul(bh, ((int64_t)1 << 62) - b61 * 2), 0x6666666666666666ll);  // beta_h (1 - beta_h)/10
+        db[2] = -fx_smul(bn * 4, 0xcccccccccccccdll);                          // -beta_n/80 (1/80 in format 62)
+    }
     a[0] = am;
     a[1] = ah;
     a[2] = an;
@@ -425,27 +474,85 @@ PIMC_HD void hh_fixed_rates(const HhFixed& c, int64_t V, int64_t a[3], int64_t l
     l[2] = an + bn;
 }
 
-// Increments dt F of one stage: K[0] of V (format 50), K[1..3] of the gates (format 59).  V (55) and the gates (61) are
-// in range on entry; false when a current leaves its format.
-PIMC_HD bool hh_fixed_stage(const HhFixed& c, const HhFixedParams& p, int64_t I45, int64_t V, const int64_t* s,
-                            int64_t* K)
+// The part of a stage that no parameter enters: the gates' increments dt F (format 59) in k[0..2], m^3 h and n^4 (format
+// 60) in k[3], k[4].  A site's parameter moves share the first stage's (the path stands still during them).
+PIMC_HD void hh_fixed_gates(const HhFixed& c, int64_t V, const int64_t* s, int64_t* k)
 {
     int64_t a[3], l[3];
-    hh_fixed_rates(c, V, a, l);
+    hh_fixed_rates<false>(c, V, a, l, nullptr, nullptr);
 #pragma unroll
-    for (int g = 0; g < 3; ++g) K[1 + g] = (a[g] >> 1) - fx_smul(l[g] * 4, s[g]);
+    for (int g = 0; g < 3; ++g) k[g] = (a[g] >> 1) - fx_smul<true>(l[g] * 4, s[g]);
     const int64_t m = s[0] * 2, h = s[1] * 2, n = s[2] * 2;  // format 62
     const int64_t m2 = fx_smul(m, m) * 4, mh = fx_smul(m, h) * 4, n2 = fx_smul(n, n) * 4;
-    const int64_t m3h = fx_smul(m2, mh), n4 = fx_smul(n2, n2);                // format 60
-    const int64_t tNa = fx_smul(V - p.ENa, (int64_t)((uint64_t)m3h << 2));    // format 53
-    const int64_t tK = fx_smul(V - p.EK, (int64_t)((uint64_t)n4 << 2));
+    k[3] = fx_smul<true>(m2, mh);
+    k[4] = fx_smul<true>(n2, n2);
+}
+
+// The increment of V, K[0] (format 50), from m^3 h and n^4; false when a term leaves its format.
+PIMC_HD bool hh_fixed_current(const HhFixedParams& p, int64_t I45, int64_t V, int64_t m3h, int64_t n4, int64_t* K)
+{
+    const int64_t tNa = fx_smul<true>(V - p.ENa, (int64_t)((uint64_t)m3h << 2));    // format 53
+    const int64_t tK = fx_smul<true>(V - p.EK, (int64_t)((uint64_t)n4 << 2));
     constexpr int64_t kTwo = 1ll << 61, kT = 1ll << 61, kS = 1ll << 59;       // 2, 256, 2^14
     const bool ok = fx_inside(m3h, kTwo) && fx_inside(n4, kTwo) && fx_inside(tNa, kT) && fx_inside(tK, kT);
-    const int64_t S = I45 - fx_smul(p.gNa, (int64_t)((uint64_t)tNa << 1)) -
-                      (fx_smul(p.gK, (int64_t)((uint64_t)tK << 1)) >> 2) - (fx_smul(p.gL, V - p.EL) >> 6);
-    K[0] = fx_smul((int64_t)((uint64_t)S << 3), p.kappa);
+    const int64_t S = I45 - fx_smul<true>(p.gNa, (int64_t)((uint64_t)tNa << 1)) -
+                      (fx_smul<true>(p.gK, (int64_t)((uint64_t)tK << 1)) >> 2) - (fx_smul<true>(p.gL, V - p.EL) >> 6);
+    K[0] = fx_smul<true>((int64_t)((uint64_t)S << 3), p.kappa);
     constexpr int64_t kK = 100ll << 50;
     return ok && fx_inside(S, kS) && fx_inside(K[0], kK);
+}
+
+// What the reverse pass of one stage takes: the Jacobian of its increments K = dt F, as doubles.
+//   kJlam: -dK_g/ds_g (3), kJgam: dK_g/dV (3), kJV: dK_0/dV, kJg: dK_0/ds_g (3), and -dK_0/dgNa, -dK_0/dgK, -dK_0/dgL,
+//   dK_0/dENa, dK_0/dEK, K_0 (dK_0/dEL = kappa gL and dK_0/dC = -K_0/C are the caller's).
+enum { kJlam = 0, kJgam = 3, kJV = 6, kJg = 7, kJp = 10, kJlen = 16 };
+
+// A stage's increments -- K[0] of V (format 50), K[1..3] of the gates (format 59) -- and its Jacobian: element j goes to J[j * stride].
+PIMC_HD bool hh_fixed_stage_adj(const HhFixed& c, const HhFixedParams& p, int64_t I45, int64_t V, const int64_t* s,
+                                int64_t* K, double* J, int stride)
+{
+    int64_t a[3], l[3], da[3], db[3];
+    hh_fixed_rates<true>(c, V, a, l, da, db);
+#pragma unroll
+    for (int g = 0; g < 3; ++g) {
+        K[1 + g] = (a[g] >> 1) - fx_smul<true>(l[g] * 4, s[g]);
+        J[(kJlam + g) * stride] = fx_double(l[g], 60);
+        J[(kJgam + g) * stride] = fx_double(da[g] - fx_smul((da[g] + db[g]) * 4, s[g]) * 2, 60);
+    }
+    const int64_t m = s[0] * 2, h = s[1] * 2, n = s[2] * 2;  // format 62
+    const int64_t m2 = fx_smul(m, m) * 4, mh = fx_smul(m, h) * 4, n2 = fx_smul(n, n) * 4;
+    const int64_t m3h = fx_smul<true>(m2, mh), n4 = fx_smul<true>(n2, n2);  // format 60
+    const int64_t m3h62 = (int64_t)((uint64_t)m3h << 2), n462 = (int64_t)((uint64_t)n4 << 2);
+    const int64_t vNa = V - p.ENa, vK = V - p.EK, vL = V - p.EL;
+    const int64_t tNa = fx_smul<true>(vNa, m3h62), tK = fx_smul<true>(vK, n462);  // format 53
+    constexpr int64_t kTwo = 1ll << 61, kT = 1ll << 61, kS = 1ll << 59, kG = 1ll << 62;
+    const int64_t kgNa57 = fx_smul(p.kappa, p.gNa), kgK59 = fx_smul(p.kappa, p.gK);  // kappa g: formats 57, 59
+    bool ok = fx_inside(m3h, kTwo) && fx_inside(n4, kTwo) && fx_inside(tNa, kT) && fx_inside(tK, kT) &&
+              fx_inside(kgNa57, kG >> 2) && fx_inside(kgK59, kG);  // kappa g below 8
+    const int64_t tNa54 = (int64_t)((uint64_t)tNa << 1), tK54 = (int64_t)((uint64_t)tK << 1);
+    const int64_t S = I45 - fx_smul<true>(p.gNa, tNa54) - (fx_smul<true>(p.gK, tK54) >> 2) - (fx_smul<true>(p.gL, vL) >> 6);
+    K[0] = fx_smul<true>((int64_t)((uint64_t)S << 3), p.kappa);
+    constexpr int64_t kK = 100ll << 50;
+    ok = ok && fx_inside(S, kS) && fx_inside(K[0], kK);
+    const int64_t kgNa = (int64_t)((uint64_t)kgNa57 << 3), kgK = (int64_t)((uint64_t)kgK59 << 1);  // format 60
+    const int64_t g1 = fx_smul(kgNa, m3h62) >> 1, g2 = fx_smul(kgK, n462) >> 1;                    // format 57
+    const int64_t g3 = fx_smul(p.kappa, p.gL) >> 5;                                                // format 57
+    J[kJV * stride] = fx_double(-(g1 + g2 + g3), 57);
+    // m^2 h, m^3 and n^3 in format 60 (below 4), times V - E: format 52, below 512 and so format 54; kappa g times that:
+    // format 50 (n: 4 times it, format 48)
+    const int64_t m2h = fx_smul(m2, h), m3 = fx_smul(m2, m), n3 = fx_smul(n2, n);
+    const int64_t tm = fx_smul(vNa, m2h * 2), th = fx_smul(vNa, m3 * 2), tn = fx_smul(vK, n3 * 2);
+    ok = ok && fx_inside(tm, kTwo) && fx_inside(th, kTwo) && fx_inside(tn, kTwo);
+    J[(kJg + 0) * stride] = fx_double(-3 * fx_smul(kgNa, (int64_t)((uint64_t)tm << 2)), 50);
+    J[(kJg + 1) * stride] = fx_double(-fx_smul(kgNa, (int64_t)((uint64_t)th << 2)), 50);
+    J[(kJg + 2) * stride] = fx_double(-fx_smul(kgK, (int64_t)((uint64_t)tn << 2)), 48);
+    J[(kJp + 0) * stride] = fx_double(fx_smul(p.kappa, tNa54), 56);
+    J[(kJp + 1) * stride] = fx_double(fx_smul(p.kappa, tK54), 56);
+    J[(kJp + 2) * stride] = fx_double(fx_smul(p.kappa, vL), 57);
+    J[(kJp + 3) * stride] = fx_double(g1, 57);
+    J[(kJp + 4) * stride] = fx_double(g2, 57);
+    J[(kJp + 5) * stride] = fx_double(K[0], 50);
+    return ok;
 }
 
 // Whether a state in fixed point is inside the range of the stage: |V| < 100, |gate| < 1.41 (their products of two stay
@@ -457,8 +564,11 @@ PIMC_HD bool hh_fixed_inside(int64_t V, const int64_t* s)
 }
 
 // One RK4 step of the HH field, f = x + (K1 + 2 K2 + 2 K3 + K4)/6, drive held at I.  False (f untouched) when a value
-// leaves the range of the formats.
-PIMC_HD bool hh_map_fixed(const HhFixed& c, const HhFixedParams& p, const double* x, double I, double* f)
+// leaves the range of the formats.  s1: the first stage's parameter-free part (hh_fixed_gates), element g at
+// s1[g * stride], taken from there (kStage1Load; written for this very x) or left there (kStage1Store) -- the same bits.
+enum { kStage1None, kStage1Store, kStage1Load };
+PIMC_HD bool hh_map_fixed(const HhFixed& c, const HhFixedParams& p, const double* x, double I, double* f,
+                          int first = kStage1None, int64_t* s1 = nullptr, int64_t stride = 0)
 {
     if (!p.ok || !fx_below(x[0], 100.0) || !fx_below(x[1], 1.375) || !fx_below(x[2], 1.375) ||
         !fx_below(x[3], 1.375) || !fx_below(I, 16384.0))
@@ -466,12 +576,24 @@ PIMC_HD bool hh_map_fixed(const HhFixed& c, const HhFixedParams& p, const double
     const int64_t V0 = fx_of(x[0], 55), I45 = fx_of(I, 45);
     int64_t s0[3], V = V0, s[3], aV = 0, as[3] = {0, 0, 0}, K[4];
     for (int g = 0; g < 3; ++g) s[g] = s0[g] = fx_of(x[1 + g], 61);
-    bool ok = true;
     // one copy of the stage's code: four would not fit the instruction cache
 #pragma unroll 1
     for (int st = 0; st < 4; ++st) {
-        ok = hh_fixed_stage(c, p, I45, V, s, K);
-        if (!ok) return false;
+        if (first == kStage1Load && st == 0) {
+#pragma unroll
+            for (int g = 0; g < 3; ++g) K[1 + g] = s1[g * stride];
+            if (!hh_fixed_current(p, I45, V, s1[3 * stride], s1[4 * stride], K)) return false;
+        } else {
+            int64_t k[5];
+            hh_fixed_gates(c, V, s, k);
+            if (first == kStage1Store && st == 0) {
+#pragma unroll
+                for (int g = 0; g < 5; ++g) s1[g * stride] = k[g];
+            }
+#pragma unroll
+            for (int g = 0; g < 3; ++g) K[1 + g] = k[g];
+            if (!hh_fixed_current(p, I45, V, k[3], k[4], K)) return false;
+        }
         const int w = (st == 1 || st == 2) ? 1 : 0, d = st < 2 ? 0 : 1;  // weight 2^w; next stage at x + K 2^(d - 1)
         aV += K[0] << w;
         V = V0 + (K[0] << (4 + d));
@@ -483,10 +605,81 @@ PIMC_HD bool hh_map_fixed(const HhFixed& c, const HhFixedParams& p, const double
         if (st < 3 && !hh_fixed_inside(V, s)) return false;
     }
     constexpr int64_t kSixth = 0x5555555555555555ll;  // 1/6, format 65
-    f[0] = fx_double(V0 + fx_smul(aV * 8, kSixth) * 2, 55);
+    f[0] = fx_double(V0 + fx_smul<true>(aV * 8, kSixth) * 2, 55);
 #pragma unroll
-    for (int g = 0; g < 3; ++g) f[1 + g] = fx_double(s0[g] + fx_smul(as[g], kSixth) * 2, 61);
+    for (int g = 0; g < 3; ++g) f[1 + g] = fx_double(s0[g] + fx_smul<true>(as[g], kSixth) * 2, 61);
     return true;
+}
+
+// The forward half of the adjoint: f as hh_map_fixed (the same bits), and the four stages' Jacobians, element j of stage
+// st at J[(st * kJlen + j) * stride].  False when a value leaves the range (f untouched, J undefined).
+PIMC_HD bool hh_map_fixed_adj(const HhFixed& c, const HhFixedParams& p, const double* x, double I, double* f, double* J,
+                              int stride)
+{
+    if (!p.ok || !fx_below(x[0], 100.0) || !fx_below(x[1], 1.375) || !fx_below(x[2], 1.375) ||
+        !fx_below(x[3], 1.375) || !fx_below(I, 16384.0))
+        return false;
+    const int64_t V0 = fx_of(x[0], 55), I45 = fx_of(I, 45);
+    int64_t s0[3], V = V0, s[3], aV = 0, as[3] = {0, 0, 0}, K[4];
+    for (int g = 0; g < 3; ++g) s[g] = s0[g] = fx_of(x[1 + g], 61);
+#pragma unroll 1
+    for (int st = 0; st < 4; ++st) {
+        if (!hh_fixed_stage_adj(c, p, I45, V, s, K, J + (int64_t)st * kJlen * stride, stride)) return false;
+        const int w = (st == 1 || st == 2) ? 1 : 0, d = st < 2 ? 0 : 1;
+        aV += K[0] << w;
+        V = V0 + (K[0] << (4 + d));
+#pragma unroll
+        for (int g = 0; g < 3; ++g) {
+            as[g] += K[1 + g] << w;
+            s[g] = s0[g] + (K[1 + g] << (1 + d));
+        }
+        if (st < 3 && !hh_fixed_inside(V, s)) return false;
+    }
+    constexpr int64_t kSixth = 0x5555555555555555ll;
+    f[0] = fx_double(V0 + fx_smul<true>(aV * 8, kSixth) * 2, 55);
+#pragma unroll
+    for (int g = 0; g < 3; ++g) f[1 + g] = fx_double(s0[g] + fx_smul<true>(as[g], kSixth) * 2, 61);
+    return true;
+}
+
+// The reverse half, in FP64: w is the cotangent of f; gx = J_x f^T w, gp += J_p f^T w (7 entries).  kgL = kappa gL,
+// iC = 1/C.  With the increments' Jacobians: u = JK^T b stage by stage from b_4 = w/6, b_3 = w/3 + u_4,
+// b_2 = w/3 + u_3/2, b_1 = w/6 + u_2/2, and gx = w + u_1 + ... + u_4.
+PIMC_HD void hh_reverse(const double* J, int stride, double kgL, double iC, const double* w, double* gx, double* gp)
+{
+    double u[4], gq[6] = {0, 0, 0, 0, 0, 0}, sb = 0.0;
+    const double sixth = 1.0 / 6.0, third = 1.0 / 3.0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        gx[a] = w[a];
+        u[a] = 0.0;
+    }
+#pragma unroll 1
+    for (int st = 3; st >= 0; --st) {
+        const double* j = J + (int64_t)st * kJlen * stride;
+        const double cw = (st == 0 || st == 3) ? sixth : third, cu = st == 2 ? 1.0 : 0.5;
+        double b[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) b[a] = fma(cu, u[a], cw * w[a]);
+        u[0] = b[0] * j[kJV * stride];
+#pragma unroll
+        for (int g = 0; g < 3; ++g) {
+            u[0] = fma(b[1 + g], j[(kJgam + g) * stride], u[0]);
+            u[1 + g] = fma(-b[1 + g], j[(kJlam + g) * stride], b[0] * j[(kJg + g) * stride]);
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) gx[a] += u[a];
+#pragma unroll
+        for (int l = 0; l < 6; ++l) gq[l] = fma(b[0], j[(kJp + l) * stride], gq[l]);
+        sb += b[0];
+    }
+    gp[0] -= gq[0];
+    gp[1] -= gq[1];
+    gp[2] -= gq[2];
+    gp[3] += gq[3];
+    gp[4] += gq[4];
+    gp[5] = fma(kgL, sb, gp[5]);
+    gp[6] = fma(-iC, gq[5], gp[6]);
 }
 
 // ---- draws -----------------------------------------------------------------------------------------------------------

@@ -191,6 +191,12 @@ __global__ void __launch_bounds__(kBlock) hmc_leap_kernel(Ctx c, HmcScalars* hs,
     __shared__ R prs[kMaxP];
     __shared__ double tot[5], kin[NP];
     __shared__ int last;
+    extern __shared__ double adj_smem[];
+    // FP64: every warp sums its share of the parameter gradients and applies
+    // the parameter move itself (70 dependent FP64 additions in one warp took
+    // 2.2 us ahead of every step's first map)
+    constexpr bool kSpread = std::is_same<R, double>::value;
+    __shared__ R sg[NP];
     const bool first = k == 0, fin = k == n_leap, ends = first || fin;
     const double fa = ends ? 0.5 : 1.0;
     const bool rk4 = c.scheme == kSchemeRK4;
@@ -203,13 +209,14 @@ __global__ void __launch_bounds__(kBlock) hmc_leap_kernel(Ctx c, HmcScalars* hs,
     pdl_trigger();
     const Coef<R> kc(c);
     // lane l < NP of warp 0 carries parameter l
+    // (FP64: of every warp)
     double p_im = 0.0, p_lo = 0.0, p_hi = 0.0;
     bool p_moving = false;
-    if (i < NP) {
-        p_im = invm[nx + i];
-        p_lo = c.st->lo[i];
-        p_hi = c.st->hi[i];
-        p_moving = (c.st->free_mask >> i) & 1u;
+    if (kSpread ? lane < NP : i < NP) {
+        p_im = invm[nx + lane];
+        p_lo = c.st->lo[lane];
+        p_hi = c.st->hi[lane];
+        p_moving = (c.st->free_mask >> lane) & 1u;
     }
     const int64_t ntile = (ld + T - 1) / T;
     // per-site data no kernel of the trajectory writes
@@ -254,7 +261,32 @@ __global__ void __launch_bounds__(kBlock) hmc_leap_kernel(Ctx c, HmcScalars* hs,
             pv[a] = owner ? V::load(P, a * ld + kk) : S{};
             em[a] = (owner && !fin) ? V::load(EM, a * ld + kk) : S{};
         }
-        if (head && wid == 0) {
+        double s_pj = 0.0, s_qp = 0.0;  // FP64: P_p(k - 3/2) and Q_p(k - 1) (k = 0: P_p(0), Q_p(0))
+        if (kSpread && head) {
+            if (lane < NP) {
+                s_pj = hs->pp[first ? 0 : (k + 1) & 1][lane];
+                s_qp = first ? Qk[nx + lane] : Qn[nx + lane];
+            }
+            // the same order of additions as one warp's: lane t adds CTAs t, t + 32, ...
+            for (int l = wid; !first && l < NP; l += NW) {
+                R t = R(0);
+                constexpr int kSumUnroll = 8;
+                for (int b0 = 0; b0 < (int)gridDim.x; b0 += 32 * kSumUnroll) {
+                    R part[kSumUnroll];
+#pragma unroll
+                    for (int u = 0; u < kSumUnroll; ++u) {
+                        const int b = b0 + 32 * u + lane;
+                        part[u] = b < (int)gridDim.x ? __ldcg((const R*)red_prev + l * kMaxGrid + b) : R(0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kSumUnroll; ++u)
+                        if (b0 + 32 * u < (int)gridDim.x) t += part[u];
+                }
+                t = warp_sum<R>(t);
+                if (lane == 0) sg[l] = t;
+            }
+        }
+        if (!kSpread && head && wid == 0) {
             // the parameters at Q_k: finish step k - 1's parameter move
             double q_l = 0.0;
             if (first) {
@@ -324,9 +356,28 @@ __global__ void __launch_bounds__(kBlock) hmc_leap_kernel(Ctx c, HmcScalars* hs,
             for (int a = 0; a < D; ++a) xs[a][T + 1] = V::x(qh[a]);
         }
         __syncthreads();
-        if (head) {
+        if (head && !kSpread) {
 #pragma unroll
             for (int l = 0; l < kMaxP; ++l) pr[l] = prs[l];
+        }
+        if (head && kSpread) {
+            if (lane < NP && !first) {
+                const double fprev = (k == 1) ? 0.5 : 1.0;
+                if (p_moving) {
+                    s_pj = s_pj - fprev * eps * (double)sg[lane];
+                    s_qp = s_qp + eps * p_im * s_pj;
+                }
+                if (blockIdx.x == 0 && wid == 0) {
+                    hs->pp[k & 1][lane] = s_pj;
+                    Qk[nx + lane] = s_qp;
+                    if (p_moving && !(s_qp >= p_lo && s_qp <= p_hi)) hs->oob = 1;
+                }
+            }
+            p_pj = s_pj;
+            double qv[kMaxP];
+#pragma unroll
+            for (int l = 0; l < kMaxP; ++l) qv[l] = __shfl_sync(kFull, s_qp, l);
+            Model::prep(qv, pr);
         }
         R own[D];
 #pragma unroll
@@ -338,7 +389,7 @@ __global__ void __launch_bounds__(kBlock) hmc_leap_kernel(Ctx c, HmcScalars* hs,
                 x[a] = xs[a][i];
                 x1[a] = xs[a][i + 1];
             }
-            term_adjoint<Model, R>(c, kc, kc.Rf, x, x1, pr, In, In1, e, own, nxt, gpl);
+            term_adjoint<Model, R>(c, kc, kc.Rf, x, x1, pr, In, In1, e, own, nxt, gpl, adj_smem + i);
 #pragma unroll
             for (int a = 0; a < D; ++a) nxs[a][i] = nxt[a];
             if (i >= 1) {
@@ -537,13 +588,13 @@ __global__ void hmc_tick_kernel(Ctx c)
 // Launch on s; with pdl, the kernel may start while the previous one on s
 // finishes (it waits in pdl_wait for that one's results).
 template <class... KArgs, class... Args>
-static cudaError_t launch_after(void (*kern)(KArgs...), unsigned grid, int block, cudaStream_t s, bool pdl,
+static cudaError_t launch_after(void (*kern)(KArgs...), unsigned grid, int block, int smem, cudaStream_t s, bool pdl,
                                 Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -580,15 +631,18 @@ static cudaError_t hmc_traj_t(const Ctx& c, const HmcBuffers& b, int n_leap, dou
     double* Qb[2] = {b.Q, b.Q2};
     hmc_begin_kernel<Model, R><<<gb, kBlock, 0, s>>>(c, b.hs, b.Q, b.P, b.EM, b.invm, eps, seed);
     cudaError_t e = cudaGetLastError();
+    constexpr int smem = adjoint_smem<Model>();
+    if (e == cudaSuccess && smem > 0)
+        e = cudaFuncSetAttribute(hmc_leap_kernel<Model, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     for (int k = 0; k <= n_leap && e == cudaSuccess; ++k)
-        e = launch_after(hmc_leap_kernel<Model, R>, gl, kBlock, s, pdl_leap, c, b.hs, Qb[k & 1], Qb[(k + 1) & 1],
+        e = launch_after(hmc_leap_kernel<Model, R>, gl, kBlock, smem, s, pdl_leap, c, b.hs, Qb[k & 1], Qb[(k + 1) & 1],
                          b.P, (const double*)b.EM, (const double*)b.invm, k, n_leap, (int)T);
     const unsigned gs = (unsigned)((c.M + 1 + kBlock - 1) / kBlock);
     if (e == cudaSuccess)
-        e = launch_after(hmc_commit_kernel<Model, R>, gs, kBlock, s, pdl, c, (const HmcScalars*)b.hs,
+        e = launch_after(hmc_commit_kernel<Model, R>, gs, kBlock, 0, s, pdl, c, (const HmcScalars*)b.hs,
                          (const double*)Qb[n_leap & 1]);
-    if (e == cudaSuccess) e = launch_after(hmc_record_kernel<Model, R>, gs, kBlock, s, pdl, c);
-    if (e == cudaSuccess) e = launch_after(hmc_tick_kernel<NP>, 1u, 1, s, pdl, c);
+    if (e == cudaSuccess) e = launch_after(hmc_record_kernel<Model, R>, gs, kBlock, 0, s, pdl, c);
+    if (e == cudaSuccess) e = launch_after(hmc_tick_kernel<NP>, 1u, 1, 0, s, pdl, c);
     return e;
 }
 

@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kBlock) grad_kernel(Ctx c, const double* Xe, c
     __shared__ double wsum[NP][kBlock / 32];
     __shared__ int last;
     __shared__ double res[NP];
+    extern __shared__ double adj_smem[];
     R pr[kMaxP], wr[kMaxD];
     Model::prep(pe ? pe : c.st->p, pr);
     const Coef<R> kc(c);
@@ -156,7 +157,7 @@ __global__ void __launch_bounds__(kBlock) grad_kernel(Ctx c, const double* Xe, c
             }
             const R In = I[k];
             const R In1 = c.scheme == kSchemeRK4 ? R(0) : I[k + 1 < c.M ? k + 1 : c.M - 1];
-            term_adjoint<Model, R>(c, kc, wr, x, x1, pr, In, In1, e, own, nxt, gpl);
+            term_adjoint<Model, R>(c, kc, wr, x, x1, pr, In, In1, e, own, nxt, gpl, adj_smem + i);
             for (int a = 0; a < D; ++a) nxs[a][i] = nxt[a];
             if (i >= 1)
                 for (int l = 0; l < NP; ++l) vp[l] += (double)gpl[l];
@@ -294,7 +295,12 @@ static cudaError_t grad_t(const Ctx& c, const double* Xe, const double* pe, doub
     T = T < 1 ? 1 : (T > kBlock - 1 ? kBlock - 1 : T);
     const int64_t ntile = (c.M + 1 + T - 1) / T;
     const unsigned grid = (unsigned)(ntile < kMaxGrid ? ntile : kMaxGrid);
-    grad_kernel<Model, R><<<grid, kBlock, 0, s>>>(c, Xe, pe, beta, gX, gp, (int)T);
+    constexpr int smem = adjoint_smem<Model>();
+    if (smem > 0) {
+        const cudaError_t e = cudaFuncSetAttribute(grad_kernel<Model, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    grad_kernel<Model, R><<<grid, kBlock, smem, s>>>(c, Xe, pe, beta, gX, gp, (int)T);
     return cudaGetLastError();
 }
 

@@ -48,6 +48,7 @@ struct pimc_handle_s {
     DevState* st = nullptr;
     double* partials = nullptr;
     unsigned long long* halo = nullptr;   // halo packets of the resident sweep
+    void* st1 = nullptr;                  // HH: first-stage values shared by a sweep's moves (absent if memory is short)
     unsigned* bar = nullptr;
     unsigned long long* flags = nullptr;  // neighbour epoch flags [2][kMaxGrid] of the sweep kernel
     uint64_t epoch = 0;                   // sweeps launched so far: the flags' epoch base
@@ -140,6 +141,9 @@ Ctx make_ctx(pimc_t h)
     c.xstride = h->grid > 100 ? 512 : 16;
     c.chk = h->chk;
     c.fx = hh_fixed_of(h->dt);
+    c.hRm = 0.5 * h->Rm;
+    for (int a = 0; a < 4; ++a) c.hRf[a] = 0.5 * h->Rf[a];
+    c.st1 = h->st1;
     return c;
 }
 
@@ -302,7 +306,7 @@ int check_finite(const double* v, int64_t n)
 
 void free_all(pimc_t h)
 {
-    void* bufs[] = {h->X, h->F[0], h->F[1], h->y, h->I, h->sig, h->acc_win, h->st, h->partials, h->halo, h->bar, h->flags,
+    void* bufs[] = {h->X, h->F[0], h->F[1], h->y, h->I, h->sig, h->acc_win, h->st, h->partials, h->halo, h->st1, h->bar, h->flags,
                     h->ticket, h->chk, h->red, h->pdraw, h->S1, h->S2, h->shift, h->hist, h->h_comp, h->h_lo, h->h_hi,
                     h->dense, h->small, h->y64, h->I64, h->trace, h->R1, h->R2, h->hmc.hs, h->hmc.Q, h->hmc.P,
                     h->hmc.Q2, h->hmc.EM, h->hmc.invm};
@@ -408,6 +412,11 @@ int pimc_create(pimc_t* out, int model, int64_t M, int D, int L, double dt, cons
             delete h;
             return r;
         }
+    }
+    // a cache only: without it every move evaluates the whole map
+    if (model == PIMC_MODEL_HH && cudaMalloc(&h->st1, sizeof(int64_t) * 5 * h->ldx) != cudaSuccess) {
+        cudaGetLastError();
+        h->st1 = nullptr;
     }
     // zeroed on the handle's stream, ahead of everything launched on it
     cudaMemsetAsync(h->bar, 0, sizeof(unsigned) * 4, h->stream);

@@ -13,14 +13,32 @@ namespace pimc {
 // kernel so the per-site code does no FP64 -> FP32 conversions.
 template <class R> struct Coef {
     R dt, Rm, Rf[kMaxD];
+    double hRm, hRf[kMaxD];  // FP64: Rm / 2 and Rf / 2 (formed per site they cost 5 FP64 instructions of 64 cycles)
     __device__ __forceinline__ explicit Coef(const Ctx& c)
     {
         dt = R(c.dt);
         Rm = R(c.Rm);
+        hRm = c.hRm;
 #pragma unroll
-        for (int a = 0; a < kMaxD; ++a) Rf[a] = R(c.Rf[a]);
+        for (int a = 0; a < kMaxD; ++a) {
+            Rf[a] = R(c.Rf[a]);
+            hRf[a] = c.hRf[a];
+        }
     }
 };
+
+// sqdiff with the weight of component a of the model error, or of the
+// measurement: the same bits in both types (halving is exact).
+template <class R> __device__ __forceinline__ R sqdiff_f(const Coef<R>& k, int a, R dp, R d)
+{
+    if constexpr (std::is_same<R, double>::value) return k.hRf[a] * (dp - d) * (dp + d);
+    else return sqdiff<R>(k.Rf[a], dp, d);
+}
+template <class R> __device__ __forceinline__ R sqdiff_m(const Coef<R>& k, R dp, R d)
+{
+    if constexpr (std::is_same<R, double>::value) return k.hRm * (dp - d) * (dp + d);
+    else return sqdiff<R>(k.Rm, dp, d);
+}
 
 // ---- scheme-generic pieces --------------------------------------------------
 // Cached value g_n of a site: the RK4 map f(x_n) (RK4 scheme, n < M) or the
@@ -64,8 +82,8 @@ __device__ __forceinline__ R eps_of(const Ctx& c, const Coef<R>& k, R xn, R xn1,
 // gp = -dt/2 (J_p F_k + J_p F_{k+1})^T w.  In, In1: the drive at t_k and at
 // t_{k+1} (the trapezoid's second vector field).
 template <class Model, class R>
-__device__ __forceinline__ void term_adjoint(const Ctx& c, const Coef<R>& kc, const R* wr, const R* x, const R* x1,
-                                             const R* pr, R In, R In1, R* e, R* own, R* nxt, R* gp)
+__device__ __forceinline__ void term_adjoint_general(const Ctx& c, const Coef<R>& kc, const R* wr, const R* x,
+                                                     const R* x1, const R* pr, R In, R In1, R* e, R* own, R* nxt, R* gp)
 {
     constexpr int D = Model::D;
     R jp[kMaxP];
@@ -108,6 +126,72 @@ __device__ __forceinline__ void term_adjoint(const Ctx& c, const Coef<R>& kc, co
         }
 #pragma unroll
         for (int l = 0; l < kMaxP; ++l) gp[l] = -(R(0.5) * kc.dt) * jp[l];
+    }
+}
+
+// The FP64 HH adjoint outside the fixed-point range (rare: one copy, called).
+static __device__ __noinline__ void hh_term_adjoint_fp64(const Ctx& c, const Coef<double>& kc, const double* wr,
+                                                         const double* x, const double* x1, const double* pr, double In,
+                                                         double In1, double* e, double* own, double* nxt, double* gp)
+{
+    term_adjoint_general<HH<double>, double>(c, kc, wr, x, x1, pr, In, In1, e, own, nxt, gp);
+}
+
+// Shared memory a CTA of kBlock threads takes for the fixed-point adjoint's
+// Jacobians (four stages a thread, [element][thread]: no bank conflicts).
+template <class Model> constexpr int adjoint_smem()
+{
+    return std::is_same<Model, HH<double>>::value ? (int)sizeof(double) * 4 * kJlen * kBlock : 0;
+}
+
+// term_adjoint_general, with FP64 HH under RK4 in fixed point: forward map and
+// the stages' Jacobians by integer arithmetic, the reverse pass in FP64 with 25
+// operations a stage instead of 85 (and the forward's exponentials).  J: the
+// thread's Jacobian slots (adjoint_smem, stride kBlock); unused otherwise.
+// Measured (M = 16384, a leapfrog step): 46 -> 25 us.
+template <class Model, class R>
+__device__ __forceinline__ void term_adjoint(const Ctx& c, const Coef<R>& kc, const R* wr, const R* x, const R* x1,
+                                             const R* pr, R In, R In1, R* e, R* own, R* nxt, R* gp, double* J)
+{
+    if constexpr (std::is_same<Model, HH<double>>::value) {
+        if (c.scheme == kSchemeRK4) {
+            double f[4], gx[4];
+            const HhFixedParams P = hh_fixed_params(c.fx, pr, kc.dt);
+            if (hh_map_fixed_adj(c.fx, P, x, In, f, J, kBlock)) {
+                double jp[7] = {0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    e[a] = x1[a] - f[a];
+                    nxt[a] = wr[a] * e[a];
+                }
+                hh_reverse(J, kBlock, kc.dt * pr[7] * pr[2], pr[7], nxt, gx, jp);
+#pragma unroll
+                for (int a = 0; a < 4; ++a) own[a] = -gx[a];
+#pragma unroll
+                for (int l = 0; l < 7; ++l) gp[l] = -jp[l];
+                return;
+            }
+        }
+        double wl[4], xl[4], x1l[4], pl[kMaxP], el[4], ol[4], nl[4], gl[kMaxP];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            wl[a] = wr[a];
+            xl[a] = x[a];
+            x1l[a] = x1[a];
+        }
+#pragma unroll
+        for (int l = 0; l < kMaxP; ++l) pl[l] = pr[l];
+        hh_term_adjoint_fp64(c, kc, wl, xl, x1l, pl, In, In1, el, ol, nl, gl);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            e[a] = el[a];
+            own[a] = ol[a];
+            nxt[a] = nl[a];
+        }
+#pragma unroll
+        for (int l = 0; l < 7; ++l) gp[l] = gl[l];
+    } else {
+        term_adjoint_general<Model, R>(c, kc, wr, x, x1, pr, In, In1, e, own, nxt, gp);
     }
 }
 

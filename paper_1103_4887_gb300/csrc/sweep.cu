@@ -265,13 +265,13 @@ __device__ __forceinline__ R site_delta(const Ctx& c, const Coef<R>& k, int64_t 
     constexpr int D = Model::D;
     R dA = R(0);
     if (n >= 1) {
-        dA += sqdiff<R>(k.Rm, xp[0] - nb.yn, x[0] - nb.yn);
+        dA += sqdiff_m<R>(k, xp[0] - nb.yn, x[0] - nb.yn);
         R dAf = R(0);
 #pragma unroll
         for (int a = 0; a < D; ++a) {
             const R e = eps_of<R>(c, k, nb.xprev[a], x[a], nb.gprev[a], nb.gcur[a]);
             const R ep = eps_of<R>(c, k, nb.xprev[a], xp[a], nb.gprev[a], gp[a]);
-            dAf += sqdiff<R>(k.Rf[a], ep, e);
+            dAf += sqdiff_f<R>(k, a, ep, e);
         }
         dA += beta * dAf;
     }
@@ -281,7 +281,7 @@ __device__ __forceinline__ R site_delta(const Ctx& c, const Coef<R>& k, int64_t 
         for (int a = 0; a < D; ++a) {
             const R e = eps_of<R>(c, k, x[a], nb.xn1[a], nb.gcur[a], nb.gn1[a]);
             const R ep = eps_of<R>(c, k, xp[a], nb.xn1[a], gp[a], nb.gn1[a]);
-            dAf += sqdiff<R>(k.Rf[a], ep, e);
+            dAf += sqdiff_f<R>(k, a, ep, e);
         }
         dA += beta * dAf;
     }
@@ -416,7 +416,7 @@ __device__ __forceinline__ R param_term(const Ctx& c, const Coef<R>& k, int64_t 
     } else {
         R t = R(0);
 #pragma unroll
-        for (int a = 0; a < D; ++a) t += beta * sqdiff<R>(k.Rf[a], xn1[a] - fp[a], xn1[a] - fc[a]);
+        for (int a = 0; a < D; ++a) t += beta * sqdiff_f<R>(k, a, xn1[a] - fp[a], xn1[a] - fc[a]);
         return t;
     }
 }
@@ -1141,6 +1141,43 @@ __device__ __forceinline__ void param_terms_paired(const Ctx& c, const Coef<floa
     bins_fold(acc, part);
 }
 
+// RK4 scheme, FP64 HH: the sites of a parameter move one a thread, as
+// param_term, with the parameters' fixed-point form made once and the first
+// stage's parameter-free part (the rates: 60 % of a stage) taken from c.st1
+// when an earlier move of the sweep left it there.  Returns whether it is there
+// now: the first executed move writes it (if its parameters are in the formats'
+// range, which is the same for every site).
+template <int NT>
+__device__ __forceinline__ bool param_terms_fixed(const Ctx& c, const Coef<double>& k, int64_t n0, int64_t nend,
+                                                  const double* pq, double beta, const double* Fc, double* Fn, bool have,
+                                                  Fix3& part)
+{
+    const double* X = (const double*)c.X;
+    const double* I = (const double*)c.I;
+    int64_t* st1 = (int64_t*)c.st1;
+    const HhFixedParams P = hh_fixed_params(c.fx, pq, k.dt);
+    for (int64_t n = n0 + threadIdx.x; n < nend; n += NT) {
+        if (!chk_site(c, 2, n)) continue;
+        double x[4], fp[4], xn1[4], fc[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            x[a] = X[a * c.ldx + n];
+            xn1[a] = X[a * c.ldx + n + 1];
+            fc[a] = Fc[a * c.ldf + n];
+        }
+        hh_map_any(c.fx, P, x, pq, I[n], k.dt, fp, have ? kStage1Load : (st1 ? kStage1Store : kStage1None), st1 + n,
+                   c.ldx);
+        double t = 0.0;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            Fn[a * c.ldf + n] = fp[a];
+            t += beta * sqdiff_f<double>(k, a, xn1[a] - fp[a], xn1[a] - fc[a]);
+        }
+        fix_add(part, t);
+    }
+    return have || (st1 && P.ok);
+}
+
 // ---- general form -----------------------------------------------------------
 
 // n_sweeps checkerboard sweeps of one chain over the sites [n0, n1) this CTA
@@ -1223,6 +1260,7 @@ __device__ void sweep_chain_general(const Ctx& c, int64_t n0, int64_t n1, int64_
         }
 
         // ---- sequential parameter moves l = 1..N_p (Sec. 4.1) ----
+        bool have_st1 = false;  // c.st1 holds this sweep's first stages
         for (int l = 0; l < NP; ++l) {
             if (!((sh.free_mask >> l) & 1u)) continue;
             if (tid == 0) sh.par_prop[l] += 1ull;
@@ -1240,6 +1278,8 @@ __device__ void sweep_chain_general(const Ctx& c, int64_t n0, int64_t n1, int64_
             if (c.scheme == kSchemeRK4) {
                 if constexpr (std::is_same<Model, HH<float>>::value)
                     param_terms_paired<NT>(c, kc, n0, nend, pq, beta, Fc, Fn, part);
+                else if constexpr (std::is_same<Model, HH<double>>::value)
+                    have_st1 = param_terms_fixed<NT>(c, kc, n0, nend, pq, beta, Fc, Fn, have_st1, part);
                 else
                     for (int64_t n = n0 + tid; n < nend; n += NT)
                         if (chk_site(c, 2, n)) fix_add(part, param_term<Model, R>(c, kc, n, pq, beta, Fc, Fn));
@@ -1533,7 +1573,8 @@ __device__ __forceinline__ void record_site(const Ctx& c, int64_t n, bool first_
 // CTA sum for both outcomes of l; after the decision warp 0 publishes the one
 // that holds.  Path and cache live in registers and shared memory for the
 // whole launch and are written back at its end.  Measured (HH, 7 free, RK4):
-// @RESIDENT_FIGURES@
+// 18.0 -> 11.2 us a sweep at M = 1024 and 18.2 -> 12.0 at M = 32768, against the
+// form that kept the path in global memory and ordered it by flags and barriers.
 template <class Model, class R, int NT, bool kTrap>
 __device__ void sweep_chain_resident(const Ctx& c, int64_t n0, int64_t n1, int64_t n_sweeps, SweepShared<R, NT>& sh,
                                      const GridSync& sync)

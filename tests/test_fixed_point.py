@@ -26,6 +26,17 @@ extern "C" int map(double dt, const double* q, const double* x, const double* I,
     }
     return c.ok;
 }
+extern "C" void adjoint(double dt, const double* q, const double* x, const double* I, const double* w, long n, double* f,
+                        double* gx, double* gp, unsigned char* ok)
+{
+    const HhFixed c = hh_fixed_of(dt);
+    for (long i = 0; i < n; ++i) {
+        double J[4 * kJlen];
+        const HhFixedParams p = hh_fixed_params(c, q + 8 * i, dt);
+        ok[i] = hh_map_fixed_adj(c, p, x + 4 * i, I[i], f + 4 * i, J, 1);
+        if (ok[i]) hh_reverse(J, 1, dt * q[8 * i + 7] * q[8 * i + 2], q[8 * i + 7], w + 4 * i, gx + 4 * i, gp + 7 * i);
+    }
+}
 extern "C" void draws(const unsigned* w, long n, double* z, double* e)
 {
     for (long i = 0; i < n; ++i) {
@@ -100,6 +111,38 @@ def test_map(lib, dt, around):
     err, half = np.abs(f - ref), np.spacing(np.abs(ref.astype(np.float64))) / 2
     assert np.all(err[0, ok] <= half[0, ok] + 2.0 ** -46)
     assert np.all(err[1:, ok] <= half[1:, ok] + 2.0 ** -56 + 2 * dt * 2.0 ** -47)
+
+
+@pytest.mark.parametrize("dt", [0.02, 0.04])
+@pytest.mark.parametrize("around", [None, -40.0, -55.0, -41.0 + 0.375, 95.0, -95.0])
+def test_adjoint(lib, dt, around):
+    """w^T J_x f and w^T J_p f against central differences in extended precision (h = 1e-5 of a scale: truncation below
+    1e-9 of the largest entry, rounding below 1e-12), and the forward half against the map, bit for bit."""
+    rng = np.random.default_rng(5)
+    n = 600
+    V = rng.uniform(-90, 60, n) if around is None else around + rng.choice([-1, 1], n) * 10.0 ** rng.uniform(-18, 0, n)
+    x = np.stack([V, rng.uniform(0, 1, n), rng.uniform(0, 0.5, n), rng.uniform(0, 0.8, n)])
+    q = NOMINAL[:, None] * rng.uniform(0.7, 1.3, (7, n))
+    I, w = rng.uniform(-20, 40, n), rng.standard_normal((4, n)) * np.array([[10.0], [100.0], [100.0], [100.0]])
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+    qa = np.ascontiguousarray(np.concatenate([q, 1.0 / q[6:7]]).T)
+    xa, wa = np.ascontiguousarray(x.T), np.ascontiguousarray(w.T)
+    f, gx, gp, ok = np.full((n, 4), np.nan), np.zeros((n, 4)), np.zeros((n, 7)), np.zeros(n, dtype=np.uint8)
+    lib.adjoint(ctypes.c_double(dt), p(qa), p(xa), p(np.ascontiguousarray(I)), p(wa), ctypes.c_long(n), p(f), p(gx), p(gp),
+                p(ok))
+    fm, okm = _call_map(lib, dt, q, x, I)
+    ok = ok.astype(bool)
+    assert not np.any(ok & ~okm) and ok.mean() > 0.5 and np.array_equal(f.T[:, ok], fm[:, ok])
+    xl, ql, Il, wl = (a.astype(L) for a in (x, q, I, w))
+    for k in range(11):
+        scale = L(1) if k < 4 else np.abs(ql[k - 4])
+        h = scale * L(1e-5)
+        d = np.zeros((11, n), dtype=L)
+        d[k] = h
+        up, dn = _map(xl + d[:4], ql + d[4:], Il, L(dt)), _map(xl - d[:4], ql - d[4:], Il, L(dt))
+        ref = ((wl * (up - dn)).sum(0) / (2 * h))[ok]
+        got = (gx[:, k] if k < 4 else gp[:, k - 4])[ok]
+        assert np.all(np.abs(got - ref) <= 1e-8 * np.abs(ref).max())
 
 
 @pytest.mark.parametrize("index,value", [(0, 100.0), (0, -1e300), (0, np.nan), (1, 1.4), (2, -np.inf), (3, np.nan)])
