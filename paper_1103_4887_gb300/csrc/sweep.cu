@@ -1639,14 +1639,30 @@ __device__ void sweep_chain_resident(const Ctx& c, int64_t n0, int64_t n1, int64
 #pragma unroll
     for (int a = 0; a < D; ++a) zn[a] = R(0);
     bool have_draws = false;
+    // sweeps until the next one that records (s >= n_init, every n_skip) or
+    // adapts (s < n_init, every n_skip): counted down, since a 64-bit remainder
+    // each sweep lies on its path
+    long long due = s0 < c.n_init ? (c.n_skip - 1) - s0 % c.n_skip
+                                  : (c.n_skip - (s0 - c.n_init) % c.n_skip) % c.n_skip;
+    // this sweep's parameter draws (warp 0), loaded a sweep ahead
+    const bool drawer = tid < NP && ((free_mask >> tid) & 1u);
+    double dz = 0.0, de = 0.0;
+    if (drawer && n_sweeps > 0) {
+        dz = __ldg(c.pdraw + 2 * tid);
+        de = __ldg(c.pdraw + 2 * tid + 1);
+    }
     for (int64_t k = 0; k < n_sweeps; ++k) {
         const long long s = s0 + k;
         const unsigned tag = (unsigned)(sh.ep0 + (unsigned long long)k + 1ull);
         // this sweep's parameter draws, evaluated before the launch by
         // param_draws_kernel (on one warp they would hold up the even phase)
-        if (tid < NP && ((free_mask >> tid) & 1u))
-            set_param_proposal<Model, R, NT>(sh, tid, __ldg(c.pdraw + 2 * (k * NP + tid)),
-                                             __ldg(c.pdraw + 2 * (k * NP + tid) + 1));
+        if (drawer) {
+            set_param_proposal<Model, R, NT>(sh, tid, dz, de);
+            if (k + 1 < n_sweeps) {
+                dz = __ldg(c.pdraw + 2 * ((k + 1) * NP + tid));
+                de = __ldg(c.pdraw + 2 * ((k + 1) * NP + tid) + 1);
+            }
+        }
         const R beta = R(sh.beta);
         R pr[kMaxP];
 #pragma unroll
@@ -1767,6 +1783,7 @@ __device__ void sweep_chain_resident(const Ctx& c, int64_t n0, int64_t n1, int64
                     if (tid < 32) cta = combine_pieces<NT>(sh, 2);
                 }
                 int buf = 0;
+                int done_l = -1, done_acc = 0;  // thread 0: a decision not yet in the chain state
                 while (true) {
                     todo &= todo - 1u;
                     const int l2 = todo ? __ffs(todo) - 1 : -1;
@@ -1776,15 +1793,25 @@ __device__ void sweep_chain_resident(const Ctx& c, int64_t n0, int64_t n1, int64
                         // thread 0: publish, wait for the total, decide
                         if (lane == 0) {
                             xch_publish(c, sync.rank, xc.round, cta);
+                            // the decision before enters the chain state while
+                            // this move's sums travel
+                            if (done_l >= 0) record_decision<R, NT>(sh, done_l, done_acc);
+                            done_l = -1;
+                            const SumWords e = sh.eword[l];
                             SumWords t;
                             bool poison;
                             if (!xch_wait(c, sync.size, xc, t, &poison)) sh.abort = 1;
                             else if (poison) {
                                 sh.slow[par] = 1;
                             } else {
-                                const int acc = words_less(t, sh.eword[l]) ? 1 : 0;
+                                const int acc = words_less(t, e) ? 1 : 0;
                                 sh.accd[par] = acc;
-                                record_decision<R, NT>(sh, l, acc);
+                                if (l2 >= 0) {
+                                    done_l = l;
+                                    done_acc = acc;
+                                } else {
+                                    record_decision<R, NT>(sh, l, acc);
+                                }
                             }
                             if (sync.lead()) chk_move(c);
                         }
@@ -1932,8 +1959,9 @@ __device__ void sweep_chain_resident(const Ctx& c, int64_t n0, int64_t n1, int64
             if (right_halo) packet_post<D, kTrap, true>(c, 1, b, tag, xr, gr);  // final for the sweep
 
             // ---- path statistics (Sec. 4.1): after N_init, every N_skip sweeps ----
-            const bool record = (s >= c.n_init) && ((s - c.n_init) % c.n_skip == 0);
-            if (record) {
+            const bool is_due = due == 0;
+            due = (s + 1 == c.n_init) ? 0 : (is_due ? c.n_skip - 1 : due - 1);
+            if (is_due && s >= c.n_init) {
                 const bool first_rec = J == 0;
                 if (own) record_site<D, kTrap>(c, n, first_rec, xr, xn, gr, gn, yv);
                 if (sync.lead() && tid < NP) accumulate(c, (int64_t)D * (M + 1) + tid, sh.p[tid], first_rec);
@@ -1956,7 +1984,7 @@ __device__ void sweep_chain_resident(const Ctx& c, int64_t n0, int64_t n1, int64
             }
 
             // ---- step-size adaptation during burn-in (Sec. 4.2) ----
-            if (s < c.n_init && ((s + 1) % c.n_skip == 0)) {
+            if (is_due && s < c.n_init) {
                 if (own) {
                     const double fac = 1.0 + c.alpha * ((double)accw / (double)c.n_skip - c.f_acc);
 #pragma unroll
