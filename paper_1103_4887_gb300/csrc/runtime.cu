@@ -282,7 +282,10 @@ void choose_grid(pimc_t h)
     if (h->grid_override > 0) {
         g = h->grid_override;
     } else {
-        const int64_t by_sm = std::min<int64_t>(h->num_sms, (sites + 63) / 64);
+        // FP32: 128 sites a CTA (one warp a scheduler, and half the CTAs in the
+        // exchange of every parameter move), FP64: 64
+        const int64_t per = h->prec == PIMC_FP64 ? 64 : 128;
+        const int64_t by_sm = std::min<int64_t>(h->num_sms, (sites + per - 1) / per);
         const int64_t by_threads = (sites + 2 * kSweepBlock - 1) / (2 * kSweepBlock);
         g = std::max<int64_t>(by_sm, by_threads);
     }
