@@ -160,6 +160,20 @@ PIMC_HD double fx_widen(float v)
 #endif
 }
 
+// The float nearest v (ties to even): results in the normal range by integer operations.
+PIMC_HD float fx_narrow(double v)
+{
+#ifdef __CUDA_ARCH__
+    const uint64_t b = (uint64_t)__double_as_longlong(v);
+    const uint32_t e = (uint32_t)(b >> 52) & 0x7ffu;
+    if (__builtin_expect(e - 897u >= 253u, 0)) return (float)v;  // below 2^-126, near overflow, or not finite
+    const uint64_t t = (b & 0x7fffffffffffffffull) + 0xfffffffull + ((b >> 29) & 1ull);
+    return __uint_as_float(((uint32_t)(t >> 29) - (896u << 23)) | ((uint32_t)(b >> 32) & 0x80000000u));
+#else
+    return (float)v;
+#endif
+}
+
 // |v| < lim for a lim whose low word is zero (false for NaN): a comparison of high words.
 PIMC_HD bool fx_below(double v, double lim)
 {

@@ -66,7 +66,7 @@ __global__ void load_refresh_kernel(Ctx c, const double* y64, const double* I64,
 template <class R>
 __device__ __forceinline__ R path_at(const Ctx& c, const double* Xe, int a, int64_t n)
 {
-    return Xe ? R(Xe[a * (c.M + 1) + n]) : ((const R*)c.X)[a * c.ldx + n];
+    return Xe ? narrow<R>(Xe[a * (c.M + 1) + n]) : ((const R*)c.X)[a * c.ldx + n];
 }
 
 // A = A_o + A_f (beta = 1): out = (A, A_o, A_f).  Per-site residuals in R,
@@ -88,7 +88,8 @@ __global__ void __launch_bounds__(kBlock) action_kernel(Ctx c, const double* Xe,
         for (int a = 0; a < D; ++a) x[a] = path_at<R>(c, Xe, a, n);
         if (n >= 1) {
             const R d = x[0] - y[n];
-            v[0] += 0.5 * c.Rm * (double)d * (double)d;
+            const double dd = widen(d);
+            v[0] += c.hRm * dd * dd;
         }
         if (n < c.M) {
             R g[D], g1[D], x1[D];
@@ -97,7 +98,8 @@ __global__ void __launch_bounds__(kBlock) action_kernel(Ctx c, const double* Xe,
             if (c.scheme != kSchemeRK4) cache_value<Model, R>(c, kc, x1, pr, n + 1, g1);
             for (int a = 0; a < D; ++a) {
                 const R e = eps_of<R>(c, kc, x[a], x1[a], g[a], g1[a]);
-                v[1] += 0.5 * c.Rf[a] * (double)e * (double)e;
+                const double ed = widen(e);
+                v[1] += c.hRf[a] * ed * ed;
             }
         }
     }
@@ -160,15 +162,15 @@ __global__ void __launch_bounds__(kBlock) grad_kernel(Ctx c, const double* Xe, c
             term_adjoint<Model, R>(c, kc, wr, x, x1, pr, In, In1, e, own, nxt, gpl, adj_smem + i);
             for (int a = 0; a < D; ++a) nxs[a][i] = nxt[a];
             if (i >= 1)
-                for (int l = 0; l < NP; ++l) vp[l] += (double)gpl[l];
+                for (int l = 0; l < NP; ++l) vp[l] += widen(gpl[l]);
         }
         __syncthreads();
         if (owner) {
             double g[D];
-            for (int a = 0; a < D; ++a) g[a] = (double)own[a];
+            for (int a = 0; a < D; ++a) g[a] = widen(own[a]);
             if (k >= 1) {
-                g[0] = c.Rm * (double)(xs[0][i] - y[k]) + g[0];
-                for (int a = 0; a < D; ++a) g[a] += (double)nxs[a][i - 1];
+                g[0] = c.Rm * widen(R(xs[0][i] - y[k])) + g[0];
+                for (int a = 0; a < D; ++a) g[a] += widen(nxs[a][i - 1]);
             }
             for (int a = 0; a < D; ++a) gX[a * ld + k] = g[a];
         }
@@ -271,16 +273,27 @@ template <class Model, class R> static cudaError_t refresh_t(const Ctx& c, cudaS
     refresh_cache_kernel<Model, R><<<(unsigned)((c.M + 1 + 255) / 256), 256, 0, s>>>(c);
     return cudaGetLastError();
 }
-static int reduce_grid(int64_t M)
+static int sm_count()
 {
-    int64_t g = (M + 1 + kBlock - 1) / kBlock;
-    if (g > kMaxGrid) g = kMaxGrid;
-    return (int)(g < 1 ? 1 : g);
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms > 0 ? sms : 1;
+}
+// CTAs of the whole-path kernels: one a tile of work, at most four an SM (what
+// their registers let run at once).  A CTA's fixed FP64 work -- parameters and
+// constants into the arithmetic type, sums of its warps, some 70 instructions a
+// warp -- is then spread over many tiles (M = 10^6, FP32-mixed: action 80 ->
+// 55 us, gradient 176 -> 98 us, against up to 4096 CTAs of two tiles).
+static int path_grid(int64_t work, int sms)
+{
+    const int64_t g = work < 4 * (int64_t)sms ? work : 4 * (int64_t)sms;
+    return (int)(g < 1 ? 1 : (g > kMaxGrid ? kMaxGrid : g));
 }
 template <class Model, class R>
 static cudaError_t action_t(const Ctx& c, const double* Xe, const double* pe, double* out, cudaStream_t s)
 {
-    action_kernel<Model, R><<<reduce_grid(c.M), kBlock, 0, s>>>(c, Xe, pe, out);
+    action_kernel<Model, R><<<path_grid((c.M + kBlock) / kBlock, sm_count()), kBlock, 0, s>>>(c, Xe, pe, out);
     return cudaGetLastError();
 }
 template <class Model, class R>
@@ -288,13 +301,11 @@ static cudaError_t grad_t(const Ctx& c, const double* Xe, const double* pe, doub
                           cudaStream_t s)
 {
     // sites a tile: spread over every SM while that leaves at most kBlock - 1 a tile
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int64_t T = (c.M + 1 + sms - 1) / (sms > 0 ? sms : 1);
+    const int sms = sm_count();
+    int64_t T = (c.M + 1 + sms - 1) / sms;
     T = T < 1 ? 1 : (T > kBlock - 1 ? kBlock - 1 : T);
     const int64_t ntile = (c.M + 1 + T - 1) / T;
-    const unsigned grid = (unsigned)(ntile < kMaxGrid ? ntile : kMaxGrid);
+    const int grid = path_grid(ntile, sms);
     constexpr int smem = adjoint_smem<Model>();
     if (smem > 0) {
         const cudaError_t e = cudaFuncSetAttribute(grad_kernel<Model, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

@@ -9,6 +9,15 @@
 
 namespace pimc {
 
+// Conversions between the arithmetic type and FP64, by integer operations: the
+// conversion instructions queue for the FP64 pipe (64 cycles a warp each), and
+// in the FP32-mixed whole-path kernels they were most of its work.
+__device__ __forceinline__ double widen(float v) { return fx_widen(v); }
+__device__ __forceinline__ double widen(double v) { return v; }
+template <class R> __device__ __forceinline__ R narrow(double v);
+template <> __device__ __forceinline__ float narrow<float>(double v) { return fx_narrow(v); }
+template <> __device__ __forceinline__ double narrow<double>(double v) { return v; }
+
 // Scalar constants of the action in the arithmetic type, formed once per
 // kernel so the per-site code does no FP64 -> FP32 conversions.
 template <class R> struct Coef {

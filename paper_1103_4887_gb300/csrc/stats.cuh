@@ -28,9 +28,6 @@ __device__ __forceinline__ void accumulate(const Ctx& c, int64_t ci, double v, b
     c.S2[ci] += d * d;
 }
 
-__device__ __forceinline__ double widen(float v) { return fx_widen(v); }
-__device__ __forceinline__ double widen(double v) { return v; }
-
 // Thread t of nt records its share; p is the current parameter vector and Fc
 // the current cache (f(x_n) or F(x_n)), which gives the model-error residuals
 // eps_{n+1} without another map evaluation; the
