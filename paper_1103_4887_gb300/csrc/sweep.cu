@@ -363,6 +363,53 @@ __device__ __forceinline__ bool site_core(const Ctx& c, const Coef<R>& k, int64_
 }
 
 // General form of a site move: operands from global memory, store on accept.
+// In two halves -- the proposal from the site's own operands, the decision from
+// its neighbours' -- so that a thread with one site can form every proposal of
+// the tile before the even decisions (an odd site's own operands stand still
+// during the even phase).
+template <class R, int D> struct SiteTrial {
+    R x[D], xp[D], gp[D], E;
+};
+
+template <class Model, class R>
+__device__ __forceinline__ void site_try(const Ctx& c, const Coef<R>& k, int64_t n, long long s, const R* pr,
+                                         SiteTrial<R, Model::D>& t)
+{
+    constexpr int D = Model::D;
+    const R* X = (const R*)c.X;
+    const R* sig = (const R*)c.sig;
+    R sg[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        t.x[a] = X[a * c.ldx + n];
+        sg[a] = sig[a * c.ldx + n];
+    }
+    const R drive = n < cache_len(c) ? ((const R*)c.I)[drive_index(c, n)] : R(0);
+    site_propose<Model, R>(c, k, n, s, pr, t.x, sg, drive, t.xp, t.gp, t.E);
+}
+
+template <class Model, class R>
+__device__ __forceinline__ bool site_finish(const Ctx& c, const Coef<R>& k, int64_t n, R beta, R* Fc,
+                                            const SiteTrial<R, Model::D>& t, unsigned long long& nonfinite)
+{
+    constexpr int D = Model::D;
+    R* X = (R*)c.X;
+    Nbhd<R, D> nb;
+    load_nbhd<Model, R>(c, n, Fc, nb);
+    const bool acc = site_decide<Model, R>(c, k, n, t.x, t.xp, t.gp, beta, t.E, nb, nonfinite);
+    if (acc) {
+#pragma unroll
+        for (int a = 0; a < D; ++a) X[a * c.ldx + n] = t.xp[a];
+        if (n < cache_len(c)) {
+#pragma unroll
+            for (int a = 0; a < D; ++a) Fc[a * c.ldf + n] = t.gp[a];
+        }
+        atomicAdd(&c.acc_win[n], 1u);
+    }
+    return acc;
+}
+
+// The whole move of one site, its operands and neighbours loaded together.
 template <class Model, class R>
 __device__ __forceinline__ bool site_move(const Ctx& c, const Coef<R>& k, int64_t n, long long s, const R* pr,
                                           R beta, R* Fc, unsigned long long& nonfinite)
@@ -1218,14 +1265,25 @@ __device__ void sweep_chain_general(const Ctx& c, int64_t n0, int64_t n1, int64_
         // tile's even flag of this sweep (its first site moved); nothing else
         // crosses a tile, so a CTA barrier ends each phase.  FP64: one copy of
         // the phase's code (the fixed-point map and draws are some 2000
-        // instructions; two copies cost instruction-cache misses).
-#pragma unroll(sizeof(R) == 8 ? 1 : 2)
+        // instructions; two copies cost instruction-cache misses), and in tiles
+        // of at most NT / 2 sites (a warp a scheduler) all proposals -- draws and
+        // maps of even and odd sites, side by side in the same warps -- ahead of
+        // the even decisions: one map's latency instead of two (M = 1000: 47.8
+        // -> 42.0 us a sweep; at 216 sites a tile, 98.5 -> 100.8, so not there).
+        constexpr bool kWide = sizeof(R) == 8;
+        const bool one = kWide && n1 - n0 <= NT / 2;
+        SiteTrial<R, D> trial;
+#pragma unroll(kWide ? 1 : 2)
         for (int parity = 0; parity < 2; ++parity) {
             unsigned n_acc = 0u, n_prop = 0u;
             R* Fc = (R*)c.F[sh.fidx];
-            const int64_t first = n0 + (((n0 & 1) != parity) ? 1 : 0);
-            for (int64_t n = first + 2 * (int64_t)tid; n < n1; n += 2 * NT) {
-                if (!chk_site(c, parity, n)) continue;
+            const int64_t first = n0 + ((!one && (n0 & 1) != parity) ? 1 : 0);
+            const int64_t step = one ? 1 : 2;
+            for (int64_t n = first + step * (int64_t)tid; n < n1; n += step * NT) {
+                const bool mine = !one || (int)(n & 1) == parity;
+                if (mine && !chk_site(c, parity, n)) continue;
+                if (kWide && (!one || parity == 0)) site_try<Model, R>(c, kc, n, s, pr, trial);
+                if (!mine) continue;
                 if constexpr (Sync::tiled) {
                     if (sync.site_flags) {
                         // the holder's warp waits as one (a lane left behind
@@ -1243,7 +1301,10 @@ __device__ void sweep_chain_general(const Ctx& c, int64_t n0, int64_t n1, int64_
                         if (!ok) continue;  // leaving: the phase's CTA barrier reads the abort
                     }
                 }
-                n_acc += site_move<Model, R>(c, kc, n, s, pr, beta, Fc, my_nf) ? 1u : 0u;
+                bool acc;
+                if constexpr (kWide) acc = site_finish<Model, R>(c, kc, n, beta, Fc, trial, my_nf);
+                else acc = site_move<Model, R>(c, kc, n, s, pr, beta, Fc, my_nf);
+                n_acc += acc ? 1u : 0u;
                 n_prop += 1u;
             }
             my_acc[0] += parity == 0 ? n_acc : 0u;
