@@ -76,7 +76,8 @@ typedef enum {
 } pimc_proposal;
 
 typedef enum {
-    PIMC_FP64 = 0,           /* every step in FP64 */
+    PIMC_FP64 = 0,           /* every step to FP64 (the HH map, its adjoint and the draws in 64-bit fixed point
+                                where their range allows: no larger errors than by FP64 instructions) */
     PIMC_FP32_MIXED = 1      /* path, cache and per-site arithmetic in FP32; the
                                 parameter-move reduction, its accept test, the
                                 global action and the moment sums in FP64 */
@@ -286,8 +287,8 @@ int pimc_accept_stats(pimc_t h, uint64_t* site_acc, uint64_t* site_prop, uint64_
 int pimc_launch_info(pimc_t h, int* grid, int* block);
 /* Form the sweep takes at the current size, precision and grid: *resident = 1
  * when every site lives in one thread for the whole launch (FP32-mixed, at
- * most 224 sites per CTA; the site phases then order on flags between
- * neighbouring CTAs), 0 for the general form (threads stride over the tile).
+ * most 224 sites per CTA; boundary sites then travel between neighbouring
+ * CTAs as words of value and epoch), 0 for the general form (threads stride over the tile).
  * Both forms give the same bits for the same tiles. */
 int pimc_sweep_form(pimc_t h, int* resident);
 /* Which forms the sweep may take: PIMC_FORM_AUTO (default; the resident form
@@ -370,8 +371,8 @@ int pimc_debug_skip_arrive(pimc_t h, int cta);
  * first rounded to FP32 when as_float != 0, computed on the current device in
  * 42-bit integer chunks of 2^-64 and rounded once to FP64; terms of magnitude
  * >= 2^62 count as infinite, NaN gives NaN.  as_float == 2 adds the FP32
- * terms through the per-thread 128-bit accumulator the parameter moves of the
- * general sweep form use (same result).  No handle; synchronous.
+ * terms through the per-thread accumulator (three 64-bit bins) the parameter
+ * moves of the general sweep form use (same result).  No handle; synchronous.
  * PIMC_ERR_ARG for n < 0 or n > 2^20, PIMC_ERR_CUDA on a device error. */
 int pimc_debug_fix_sum(const double* terms, int64_t n, int as_float, double* out);
 /* Throughput probe of the model map f (the RK4 map of Eq. (action)'s

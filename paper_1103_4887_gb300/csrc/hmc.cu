@@ -632,8 +632,6 @@ static cudaError_t hmc_traj_t(const Ctx& c, const HmcBuffers& b, int n_leap, dou
     hmc_begin_kernel<Model, R><<<gb, kBlock, 0, s>>>(c, b.hs, b.Q, b.P, b.EM, b.invm, eps, seed);
     cudaError_t e = cudaGetLastError();
     constexpr int smem = adjoint_smem<Model>();
-    if (e == cudaSuccess && smem > 0)
-        e = cudaFuncSetAttribute(hmc_leap_kernel<Model, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     for (int k = 0; k <= n_leap && e == cudaSuccess; ++k)
         e = launch_after(hmc_leap_kernel<Model, R>, gl, kBlock, smem, s, pdl_leap, c, b.hs, Qb[k & 1], Qb[(k + 1) & 1],
                          b.P, (const double*)b.EM, (const double*)b.invm, k, n_leap, (int)T);
@@ -644,6 +642,12 @@ static cudaError_t hmc_traj_t(const Ctx& c, const HmcBuffers& b, int n_leap, dou
     if (e == cudaSuccess) e = launch_after(hmc_record_kernel<Model, R>, gs, kBlock, 0, s, pdl, c);
     if (e == cudaSuccess) e = launch_after(hmc_tick_kernel<NP>, 1u, 1, 0, s, pdl, c);
     return e;
+}
+
+cudaError_t prepare_hmc()
+{
+    return cudaFuncSetAttribute(hmc_leap_kernel<HH<double>, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                adjoint_smem<HH<double>>());
 }
 
 cudaError_t launch_hmc_trajectory(int model, int prec, const Ctx& c, const HmcBuffers& b, int n_leap, double eps,

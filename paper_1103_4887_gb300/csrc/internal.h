@@ -74,6 +74,7 @@ struct Ctx {
     int64_t wait_ns;
     int skip_cta;
     int64_t tile;                 // sites per CTA in the sweep kernel
+    int num_sms;                  // SMs of the handle's device
     HhFixed fx;                   // constants of dt of the fixed-point FP64 HH map
     double hRm, hRf[4];           // Rm / 2, Rf / 2
     void* st1;                    // HH: first-stage values of the sites, shared by a sweep's parameter moves --
@@ -153,6 +154,10 @@ cudaError_t launch_param_delta(int model, int prec, const Ctx& c, int l, double 
 cudaError_t launch_fix_sum(const double* t, int64_t n, int as_float, double* out, cudaStream_t s);
 cudaError_t launch_lane_maps(const double* X, const double* I, const double* p, double dt, int64_t n, double* out,
                              unsigned* mismatch, cudaStream_t s);
+// Opt the FP64 HH adjoint kernels in to their shared memory on the current
+// device (once a handle, at its creation).
+cudaError_t prepare_grad();
+cudaError_t prepare_hmc();
 // dst[i] = (storage type) src[i], i < n.
 cudaError_t launch_convert(int prec, const double* src, void* dst, int64_t n, cudaStream_t s);
 // Ensemble forecast from the current state: out[e][a][k] (device, FP64).

@@ -273,13 +273,6 @@ template <class Model, class R> static cudaError_t refresh_t(const Ctx& c, cudaS
     refresh_cache_kernel<Model, R><<<(unsigned)((c.M + 1 + 255) / 256), 256, 0, s>>>(c);
     return cudaGetLastError();
 }
-static int sm_count()
-{
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 1;
-}
 // CTAs of the whole-path kernels: one a tile of work, at most four an SM (what
 // their registers let run at once).  A CTA's fixed FP64 work -- parameters and
 // constants into the arithmetic type, sums of its warps, some 70 instructions a
@@ -293,7 +286,7 @@ static int path_grid(int64_t work, int sms)
 template <class Model, class R>
 static cudaError_t action_t(const Ctx& c, const double* Xe, const double* pe, double* out, cudaStream_t s)
 {
-    action_kernel<Model, R><<<path_grid((c.M + kBlock) / kBlock, sm_count()), kBlock, 0, s>>>(c, Xe, pe, out);
+    action_kernel<Model, R><<<path_grid((c.M + kBlock) / kBlock, c.num_sms), kBlock, 0, s>>>(c, Xe, pe, out);
     return cudaGetLastError();
 }
 template <class Model, class R>
@@ -301,21 +294,22 @@ static cudaError_t grad_t(const Ctx& c, const double* Xe, const double* pe, doub
                           cudaStream_t s)
 {
     // sites a tile: spread over every SM while that leaves at most kBlock - 1 a tile
-    const int sms = sm_count();
+    const int sms = c.num_sms;
     int64_t T = (c.M + 1 + sms - 1) / sms;
     T = T < 1 ? 1 : (T > kBlock - 1 ? kBlock - 1 : T);
     const int64_t ntile = (c.M + 1 + T - 1) / T;
     const int grid = path_grid(ntile, sms);
-    constexpr int smem = adjoint_smem<Model>();
-    if (smem > 0) {
-        const cudaError_t e = cudaFuncSetAttribute(grad_kernel<Model, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-    }
-    grad_kernel<Model, R><<<grid, kBlock, smem, s>>>(c, Xe, pe, beta, gX, gp, (int)T);
+    grad_kernel<Model, R><<<grid, kBlock, adjoint_smem<Model>(), s>>>(c, Xe, pe, beta, gX, gp, (int)T);
     return cudaGetLastError();
 }
 
 
+
+cudaError_t prepare_grad()
+{
+    return cudaFuncSetAttribute(grad_kernel<HH<double>, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                adjoint_smem<HH<double>>());
+}
 
 cudaError_t launch_init_path(int model, int prec, const Ctx& c, cudaStream_t s) { PIMC_DISPATCH(init_t, c, s); }
 cudaError_t launch_refresh_cache(int model, int prec, const Ctx& c, cudaStream_t s)

@@ -140,6 +140,7 @@ Ctx make_ctx(pimc_t h)
     // (probe: 0.67 us against 0.84 at 16 CTAs, 1.08 against 0.89 at 152)
     c.xstride = h->grid > 100 ? 512 : 16;
     c.chk = h->chk;
+    c.num_sms = h->num_sms;
     c.fx = hh_fixed_of(h->dt);
     c.hRm = 0.5 * h->Rm;
     for (int a = 0; a < 4; ++a) c.hRf[a] = 0.5 * h->Rf[a];
@@ -370,6 +371,8 @@ int pimc_create(pimc_t* out, int model, int64_t M, int D, int L, double dt, cons
     h->ldf = round_up(M + 1, 64);
     cudaError_t e = cudaGetDevice(&h->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (e == cudaSuccess && model == PIMC_MODEL_HH) e = prepare_grad();
+    if (e == cudaSuccess && model == PIMC_MODEL_HH) e = prepare_hmc();
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         int r = fail(nullptr, PIMC_ERR_CUDA, "device setup: %s", cudaGetErrorString(e));

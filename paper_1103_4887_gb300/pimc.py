@@ -166,7 +166,7 @@ def action_static(model, M, dt, Rm, Rf, X_ptr, p_ptr, y_ptr, I_ptr, out_ptr, str
 
 def debug_fix_sum(terms, as_float=False, acc128=False):
     """The exact sum parameter moves use, applied to a host array (test hook);
-    acc128: FP32 terms through the general form's 128-bit per-thread sum."""
+    acc128: FP32 terms through the general form's per-thread bins."""
     L = load()
     t = _f64(terms)
     out = np.zeros(1)

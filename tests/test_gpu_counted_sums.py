@@ -45,3 +45,35 @@ def test_sums_out_of_range(precision, scale, M):
             assert np.array_equal(np.asarray(x), np.asarray(y), equal_nan=True)
         assert all(np.array_equal(x, y) for x, y in zip(s.accept_stats(), ref.accept_stats()))
     b.close()
+
+
+@pytest.mark.parametrize("scheme", [0, 1])
+@pytest.mark.parametrize("M,grid", [(12, 6), (15, 8), (255, 2), (447, 2), (300, 3)])
+def test_tile_edges(M, grid, scheme):
+    """Tiles of one site, of two, of the resident form's largest size and ragged last ones: boundary sites by packets
+    (resident), by flags (general) and in one CTA, over burn-in with adaptation and annealing, then recording, in three
+    launches."""
+    prob = synth.hh_problem(M, data_seed=8, free="all")
+    prob.scheme = scheme
+    got = []
+    for form in ("auto", "general", "batch"):
+        s = pimc.Sampler.from_problem(prob, precision=pimc.FP32_MIXED)
+        if form != "batch":
+            s.set_grid(grid)
+            s.set_sweep_form(form)
+            assert s.sweep_form() == ("resident" if form == "auto" else "general") and s.launch_info()[0] > 1
+        s.set_schedule(n_init=7, n_skip=3, beta0=0.3, n_cool=5, f_acc=0.4, alpha=0.3)
+        s.set_param_trace(40)
+        run = s
+        if form == "batch":
+            run = pimc.Batch([s])
+            run.set_tuning(256, 1, 1)
+        for n in (5, 1, 17):
+            run.sweep(n, 23)
+        got.append((*s.state(), *s.moments(), *s.residual_moments(), s.param_trace(), *s.steps(), *s.accept_stats(),
+                    np.array(s.sweep_counter())))
+        if form == "batch":
+            run.close()
+    for other in got[1:]:
+        for x, y in zip(got[0], other):
+            assert np.array_equal(np.asarray(x), np.asarray(y), equal_nan=True)
