@@ -192,10 +192,12 @@ __global__ void __launch_bounds__(kBlock) hmc_leap_kernel(Ctx c, HmcScalars* hs,
     __shared__ double tot[5], kin[NP];
     __shared__ int last;
     extern __shared__ double adj_smem[];
-    // FP64: every warp sums its share of the parameter gradients and applies
-    // the parameter move itself (70 dependent FP64 additions in one warp took
-    // 2.2 us ahead of every step's first map)
-    constexpr bool kSpread = std::is_same<R, double>::value;
+    // FP64, many parameters: every warp sums its share of the parameter
+    // gradients and applies the parameter move itself (70 dependent FP64
+    // additions in one warp took 2.2 us ahead of every step's first map).
+    // With one or two of them one warp's sums hide behind the others' position
+    // updates (one parameter, M = 200: spread 9.8 us a step, one warp 9.3).
+    constexpr bool kSpread = std::is_same<R, double>::value && NP > 2;
     __shared__ R sg[NP];
     const bool first = k == 0, fin = k == n_leap, ends = first || fin;
     const double fa = ends ? 0.5 : 1.0;
@@ -209,7 +211,7 @@ __global__ void __launch_bounds__(kBlock) hmc_leap_kernel(Ctx c, HmcScalars* hs,
     pdl_trigger();
     const Coef<R> kc(c);
     // lane l < NP of warp 0 carries parameter l
-    // (FP64: of every warp)
+    // (spread: of every warp)
     double p_im = 0.0, p_lo = 0.0, p_hi = 0.0;
     bool p_moving = false;
     if (kSpread ? lane < NP : i < NP) {
@@ -261,7 +263,7 @@ __global__ void __launch_bounds__(kBlock) hmc_leap_kernel(Ctx c, HmcScalars* hs,
             pv[a] = owner ? V::load(P, a * ld + kk) : S{};
             em[a] = (owner && !fin) ? V::load(EM, a * ld + kk) : S{};
         }
-        double s_pj = 0.0, s_qp = 0.0;  // FP64: P_p(k - 3/2) and Q_p(k - 1) (k = 0: P_p(0), Q_p(0))
+        double s_pj = 0.0, s_qp = 0.0;  // spread: P_p(k - 3/2) and Q_p(k - 1) (k = 0: P_p(0), Q_p(0))
         if (kSpread && head) {
             if (lane < NP) {
                 s_pj = hs->pp[first ? 0 : (k + 1) & 1][lane];
