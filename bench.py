@@ -53,10 +53,10 @@ KERNEL_SOURCES = ("paper_1103_4887_gb300/csrc/sweep.cu", "paper_1103_4887_gb300/
                   "paper_1103_4887_gb300/csrc/internal.h")
 TRAFFIC = {
     # one 10-sweep bench step of sweep_resident_kernel<HH<float>>, M = 32768
-    ("resident", 32768): {"bytes": 7.8523e6, "sweeps": 10, "src": "3933e0b65b73c5e5",
+    ("resident", 32768): {"bytes": 7.8418e6, "sweeps": 10, "src": "c2e9299b5e033110",
                           "profile": "profiles/sweep_resident_kernel_hh_M32768_full.md"},
     # one 10-sweep launch of sweep_kernel<HH<float>,float>, M = 2^20
-    ("general", 1048576): {"bytes": 586.50e6, "sweeps": 10, "src": "3933e0b65b73c5e5",
+    ("general", 1048576): {"bytes": 670.07e6, "sweeps": 10, "src": "c2e9299b5e033110",
                            "profile": "profiles/sweep_kernel_hh_M1048576_full.md"},
 }
 
@@ -294,7 +294,7 @@ def map_ceiling():
             r = pimc.debug_map_rate(packed, k, 4000)
             out[f"{'packed' if packed else 'single'}_{k}cta_per_sm"] = {"maps_per_s": r, "frac_of_derived_peak":
                                                                          r / peak_maps}
-    # the FP64 map (software exponentials on the FP64 pipe), the plain sweep's ceiling
+    # the FP64 map (fixed point on the integer pipe), the plain sweep's ceiling
     out["fp64_1cta_per_sm"] = {"maps_per_s": pimc.debug_map_rate(False, 1, 200, fp64=True)}
     return out
 
@@ -345,10 +345,10 @@ def sweep_M_rows(exps=range(10, 21, 2), cpu_budget_s=4.0, ceiling=None):
                     entry["traffic_bytes_per_10_sweeps"] = tr
                     entry["dram_gbs"] = tr / (10 * ms * 1e-3) / 1e9
             else:
-                # FP64 transcendental functions are software sequences on the FP64
-                # pipe: the achieved rate is stated as maps/s against the FP64 map's
-                # own measured ceiling; the FP32 count does not apply
-                entry["note"] = "FP64 pipe-bound (software exp); compare maps/s"
+                # the FP64 map runs in fixed point on the integer pipe: the achieved
+                # rate is stated as maps/s against the FP64 map's own measured
+                # ceiling; the FP32 count does not apply
+                entry["note"] = "integer-pipe-bound (map in fixed point); compare maps/s"
                 if ceiling and "fp64_1cta_per_sm" in ceiling:
                     entry["frac_of_fp64_map_ceiling"] = (maps / (ms * 1e-3)) / ceiling["fp64_1cta_per_sm"]["maps_per_s"]
             row[name] = entry
