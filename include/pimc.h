@@ -327,16 +327,20 @@ int pimc_batch_sync(pimc_batch_t b);
  * least 2 * threads_per_cta sites each), run together by as many CTAs of the
  * launch, which synchronise on the chain's own barrier word and exact-sum
  * slots with bounded waits (the launch is then cooperative); 1 keeps every
- * chain whole.  A chain's results do not depend on the tile shape.
- * PIMC_ERR_ARG for values out of range. */
+ * chain whole.  Without this call (or a cached choice of the autotuner), a batch
+ * of fewer chains than the device holds CTAs is cut into tiles where that
+ * shortens the sweep, one tile a CTA.  A chain's results do not depend on the
+ * tile shape.  PIMC_ERR_ARG for values out of range. */
 int pimc_batch_set_tuning(pimc_batch_t b, int threads_per_cta, int ctas_per_sm, int ctas_per_chain);
 /* The current plan: CTAs of a launch, threads per CTA, chains split over
  * several CTAs (any output may be NULL). */
 int pimc_batch_info(pimc_batch_t b, int* n_ctas, int* threads_per_cta, int* n_split);
 /* Time trial_sweeps real sweeps (they advance every chain: run this during
  * burn-in) for each tile shape -- threads per CTA x CTAs per SM x CTAs per
- * long chain (1, 2, 4) -- and keep the fastest; the choice is cached per
- * process for batches of the same model, precision, size and chain count. */
+ * long chain (1, 2, 4, and the plan of a batch without tuning, for which
+ * *ctas_per_chain is the largest of 1, 2, 4 not above the most tiles that plan
+ * gives a chain) -- and keep the fastest;
+ * the choice is cached per process for batches of the same model, precision, size and chain count. */
 int pimc_batch_autotune(pimc_batch_t b, int64_t trial_sweeps, uint64_t seed, int* threads_per_cta, int* ctas_per_sm,
                         int* ctas_per_chain);
 

@@ -8,6 +8,7 @@
 #include <cstddef>
 #include <map>
 #include <memory>
+#include <numeric>
 #include <queue>
 #include <cstdio>
 #include <cstring>
@@ -1402,8 +1403,9 @@ struct pimc_batch_s {
     int* d_first = nullptr;
     BatchItem* d_items = nullptr;
     int n_ctas = 0, nt = 256, ctas_per_sm = 0;
-    int split = 1;          // most CTAs one chain may be split over
+    int split = 0;          // most CTAs one chain may be split over (0: spread_tiles decides)
     int n_split = 0;        // chains split over several CTAs in the current plan
+    int max_tiles = 1;      // most tiles of a chain in it
     std::vector<unsigned> versions;
     cudaGraphExec_t exec = nullptr;
     int64_t graph_sweeps = -1;
@@ -1442,6 +1444,52 @@ double chain_cost(pimc_t h)
     return (double)(h->M + 1) * (double)(1 + nf);
 }
 
+// Tiles of every chain when nothing was asked for and the chains are fewer than
+// the CTAs that can be resident: as many as make the longest tile shortest with
+// one tile a CTA.  Empty where whole chains are the better plan: a tile's moves
+// and phases wait for the chain's other CTAs (about 9 us a sweep in all, HH with 3
+// free parameters), which an FP32 HH sweep spends on 600 sites, one of the cheap
+// models on 1400, an FP64 one on 80, and two CTAs an SM slow each other.  So the
+// longest tile has to be at most 0.6 of the longest chain and shorter by twice
+// that many sites (FP64: by one tile's least size).  Measured, us a sweep of HH,
+// whole chains -> tiles: FP32 16 x 16384 261 -> 38, 64 x 16384 289 -> 118,
+// 64 x 4096 (7 free) 122 -> 73, 16 x 2048 39 -> 27, 128 x 4096 76 -> 67; left
+// whole: 16 x 1200 (26.6, 27.8), 128 x 1024 (22.8, 30.4), 200 x 4096 (101, 120);
+// FP64 16 x 16384 2489 -> 369, 64 x 4096 (7 free) 1181 -> 710.
+std::vector<int> spread_tiles(pimc_batch_t b, const std::vector<double>& cost, int slots)
+{
+    const int n = (int)b->hs.size();
+    if (n >= slots) return {};
+    std::vector<int64_t> most(n);
+    int longest = 0;
+    double hi = 0.0;
+    for (int i = 0; i < n; ++i) {
+        most[i] = std::min<int64_t>(64, std::max<int64_t>(1, (b->hs[i]->M + 1) / (2 * b->nt)));
+        if (cost[i] > hi) {
+            hi = cost[i];
+            longest = i;
+        }
+    }
+    const auto tiles = [&](int i, double len) { return std::min(most[i], std::max<int64_t>(1, (int64_t)std::ceil(cost[i] / len))); };
+    // the shortest tile cost that fits (one tile a chain always does)
+    double lo = 0.0, len = hi;
+    for (int it = 0; it < 40; ++it) {
+        const double mid = 0.5 * (lo + len);
+        int64_t sum = 0;
+        for (int i = 0; i < n; ++i) sum += tiles(i, mid);
+        if (sum <= slots) len = mid;
+        else lo = mid;
+    }
+    double part = 0.0;  // longest tile
+    for (int i = 0; i < n; ++i) part = std::max(part, cost[i] / (double)tiles(i, len));
+    const bool heavy = b->model == PIMC_MODEL_HH || b->model == PIMC_MODEL_HH_PAPER;
+    const double saved = (double)(b->hs[longest]->M + 1) * (1.0 - part / hi);
+    if (part > 0.6 * hi || saved < (b->prec == PIMC_FP64 ? 2.0 * b->nt : heavy ? 1024.0 : 2048.0)) return {};
+    std::vector<int> g(n);
+    for (int i = 0; i < n; ++i) g[i] = (int)tiles(i, len);
+    return g;
+}
+
 // Contexts of all chains and their assignment to CTAs, longest first.  With
 // split > 1, a chain costing more than the mean load of a CTA is cut into up
 // to `split` tiles (at least 2 nt sites each), which go to that many of the
@@ -1461,6 +1509,10 @@ int batch_build(pimc_batch_t b)
     for (int i = 0; i < n; ++i) total += (cost[i] = chain_cost(b->hs[i]));
     // enough CTAs for every chain, or for every tile when chains are split
     b->n_ctas = std::max(1, std::min(b->split > 1 ? per_sm * sms : n, per_sm * sms));
+    std::vector<int> spread;
+    if (b->split == 0) spread = spread_tiles(b, cost, per_sm * sms);
+    if (!spread.empty()) b->n_ctas = std::accumulate(spread.begin(), spread.end(), 0);
+    b->max_tiles = 1;
     std::vector<Ctx> ctx(n);
     std::vector<int> idx(n);
     for (int i = 0; i < n; ++i) {
@@ -1475,7 +1527,7 @@ int batch_build(pimc_batch_t b)
     std::vector<int> by_load(b->n_ctas);
     b->n_split = 0;
     for (int i : idx) {
-        int g = 1;
+        int g = spread.empty() ? 1 : spread[i];
         if (b->split > 1 && cost[i] > target) {
             const int64_t max_tiles = std::max<int64_t>(1, (b->hs[i]->M + 1) / (2 * b->nt));
             g = (int)std::min<int64_t>({(int64_t)b->split, (int64_t)std::ceil(cost[i] / target), max_tiles,
@@ -1491,6 +1543,7 @@ int batch_build(pimc_batch_t b)
             load[by_load[r]] += cost[i] / g;
         }
         if (g > 1) b->n_split++;
+        b->max_tiles = std::max(b->max_tiles, g);
     }
     std::vector<int> first(b->n_ctas + 1, 0);
     std::vector<BatchItem> items;
@@ -1686,17 +1739,17 @@ int pimc_batch_autotune(pimc_batch_t b, int64_t trial_sweeps, uint64_t seed, int
     float best = 1e30f;
     Tuning best_t{b->nt, b->ctas_per_sm, b->split};
     const int nts[2] = {128, 256};
-    const int splits[3] = {1, 2, 4};
+    const int splits[4] = {1, 2, 4, 0};
     for (int ni = 0; ni < 2; ++ni) {
         const int occ = batch_ctas_per_sm(b->model, b->prec, nts[ni]);
         for (int k = 1; k <= occ; k *= 2) {
-            for (int si = 0; si < 3; ++si) {
+            for (int si = 0; si < 4; ++si) {
                 b->nt = nts[ni];
                 b->ctas_per_sm = k;
                 b->split = splits[si];
                 int r = batch_build(b);
                 if (r != PIMC_OK) return r;
-                if (splits[si] > 1 && b->n_split == 0) continue;  // nothing to split: same as split 1
+                if (splits[si] != 1 && b->n_split == 0) continue;  // nothing to split: same as split 1
                 BCK(b, cudaEventRecord(e0, b->stream));
                 BCK(b, batch_launch(b, trial_sweeps, seed));
                 BCK(b, cudaEventRecord(e1, b->stream));
@@ -1718,8 +1771,9 @@ int pimc_batch_autotune(pimc_batch_t b, int64_t trial_sweeps, uint64_t seed, int
     tune_cache()[std::make_pair(tune_key_sites(b), (int)b->hs.size())] = best_t;
     if (threads_per_cta) *threads_per_cta = best_t.nt;
     if (ctas_per_sm) *ctas_per_sm = best_t.ctas_per_sm;
-    if (ctas_per_chain) *ctas_per_chain = best_t.split;
-    return batch_build(b);
+    const int r = batch_build(b);
+    if (ctas_per_chain) *ctas_per_chain = best_t.split ? best_t.split : (b->max_tiles >= 4 ? 4 : b->max_tiles >= 2 ? 2 : 1);
+    return r;
 }
 
 }  // extern "C"
