@@ -887,23 +887,26 @@ __device__ __forceinline__ SumWords words_of(const Fix3& f)
 }
 
 // An FP32 term t in the fixed point of the exact sums, as four signed pieces of
-// 24 bits (T = sum_j p_j 2^(24 j)), whose 32-lane and 8-warp sums fit 32 bits;
-// the same truncation toward zero as fix_add.  False (pieces zero) when |t| >=
-// 2^31 or not finite.
+// 23 bits (T = sum_j p_j 2^(23 j)); the same truncation toward zero as fix_add.
+// A tile's sum of pieces has to fit 32 bits: at most 224 site threads of
+// magnitudes up to 2^23 - 1, below 2^30.81 (24-bit pieces would reach 2^31.81 and
+// wrap from 129 terms of one sign and binade on).  False (pieces zero) when
+// |t| >= 2^28 or not finite.
+constexpr int kPieceBits = 23;
 __device__ __forceinline__ bool term_pieces(float t, int p[4])
 {
     const unsigned b = __float_as_uint(t);
     const unsigned ex = (b >> 23) & 0xffu;
     int sh = (ex ? (int)ex - 150 : -149) + 64;  // bit of T that the mantissa's bit 0 lands on
-    const bool ok = sh <= 71;                   // also false for infinities and NaN (sh = 169)
+    const bool ok = sh <= 68;                   // also false for infinities and NaN (sh = 169)
     unsigned man = ok ? (ex ? (b & 0x7fffffu) | 0x800000u : (b & 0x7fffffu)) : 0u;
     if (sh < 0) {
         man = sh > -24 ? man >> -sh : 0u;
         sh = 0;
     }
-    const int idx = (sh * 2731) >> 16, off = sh - 24 * idx;  // sh / 24, sh % 24 (sh <= 71)
-    const unsigned long long v = (unsigned long long)man << off;
-    int lo = (int)((unsigned)v & 0xffffffu), hi = (int)(unsigned)(v >> 24);
+    const int idx = (sh * 2850) >> 16, off = sh - kPieceBits * idx;  // sh / 23, sh % 23 (sh <= 68)
+    const unsigned long long v = (unsigned long long)man << off;     // below 2^46: two pieces
+    int lo = (int)((unsigned)v & ((1u << kPieceBits) - 1u)), hi = (int)(unsigned)(v >> kPieceBits);
     if (b >> 31) {
         lo = -lo;
         hi = -hi;
@@ -1551,7 +1554,7 @@ __device__ __forceinline__ void warp_pieces(SweepShared<float, NT>& sh, int o, c
 }
 
 // The CTA sum of one outcome's pieces (one whole warp; all lanes get it).
-// Warp 0 holds no site.
+// Warp 0 holds no site, so seven warps' sums add up, within 32 bits.
 template <int NT>
 __device__ __forceinline__ SumWords combine_pieces(const SweepShared<float, NT>& sh, int o)
 {
@@ -1565,10 +1568,12 @@ __device__ __forceinline__ SumWords combine_pieces(const SweepShared<float, NT>&
     long long p[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) p[j] = (long long)__shfl_sync(kAll, v, j);
-    const long long lo = p[0] + p[1] * (1ll << 24), hi = p[2] + p[3] * (1ll << 24);  // T = lo + hi 2^48
-    SumWords t;
+    static_assert((NT - 32) * ((1ll << kPieceBits) - 1) < (1ll << 31), "the sum of a tile's pieces fits 32 bits");
+    const long long lo = p[0] + p[1] * (1ll << kPieceBits), hi = p[2] + p[3] * (1ll << kPieceBits);
+    SumWords t;  // T = lo + hi 2^46
+    static_assert(2 * kPieceBits == kSumLow + 1, "hi's weight is twice H's");
     t.L = (unsigned long long)lo & ((1ull << kSumLow) - 1ull);
-    t.H = (lo >> kSumLow) + hi * 8;
+    t.H = (lo >> kSumLow) + hi * 2;
     if (bad || hi <= -(1ll << 40) || hi >= (1ll << 40) || t.H <= -kSumLimit || t.H >= kSumLimit) {
         t.L = 0ull;
         t.H = kSumPoison;
