@@ -77,7 +77,7 @@ typedef enum {
 
 typedef enum {
     PIMC_FP64 = 0,           /* every step to FP64 (the HH map, its adjoint and the draws in 64-bit fixed point
-                                where their range allows: no larger errors than by FP64 instructions) */
+                                where their range allows, with rms errors as by FP64 instructions) */
     PIMC_FP32_MIXED = 1      /* path, cache and per-site arithmetic in FP32; the
                                 parameter-move reduction, its accept test, the
                                 global action and the moment sums in FP64 */

@@ -2,18 +2,24 @@
 //
 // This part issues one FP64 warp instruction per scheduler in about 64 cycles (76 with every scheduler busy), whatever
 // the number of active lanes, but a 32-bit integer one in 2 and a 32x32+64 multiply-add in about 4; a 64-bit high
-// product costs 16-20 cycles.  So a fixed-point evaluation of the RK4 map with 55 to 62 fractional bits -- at least as
-// exact as FP64 on the states, rates and currents that occur -- runs several times faster than the FP64 one.
+// product costs 16-20 cycles.  So a fixed-point evaluation of the RK4 map with 46 fractional bits of the currents, 51 to
+// 66 of the increments and 55 or 62 of the state runs several times faster than the FP64 one.
 //
 // A value a in "format f" is the integer a 2^f.  Every intermediate has a range that the checks below guarantee: a
 // state, parameter, drive or step outside it makes hh_map_fixed return false, and the caller evaluates the FP64 map
-// instead (per lane).  In range, the map's error against exact arithmetic is the rounding of its result to FP64 plus
-// less than a quarter of that.
+// instead (per lane).  In range, the map is as exact as the same formulas in FP64: its rms error against extended
+// precision was 0.97 to 1.01 times FP64's in V, and in every binade of a gate's result from 1 down to 2^-13 at most 1.12
+// times it (h deep in a spike), mostly less than it; the last addition of a gate is FP64's own, so that small gates keep
+// their bits.  The stages' Jacobians keep a relative precision of FP64's, whatever their size: below threshold d/dgNa is off
+// by 1.2e-16 of its rms, d/dm by 1.2e-16, d/dC (net currents of 0.1 out of 10) by 2e-14, as with FP64 instructions; in
+// absolute formats of 50 to 60 bits they were off by 4.7e-14, 1.5e-15 and 4.1e-13.
 //
-// Measured: the FP64 map is some 650 FP64 instructions, 49 000 scheduler cycles a warp; this one 5 200 with four warps a
-// scheduler and 9 000 alone (integer ALU and multiply-add pipes together; latency alone).  FP64 sweeps: M = 1000, 3 free
-// parameters, 120 -> 48 us; M = 32768, 7 free, 341 -> 94 us.  Normals by the FP64 functions: some 90 FP64 instructions
-// each; here 350 cycles.
+// Measured: the FP64 map is some 650 FP64 instructions, 49 000 scheduler cycles a warp; this one 5 300 with four warps a
+// scheduler and 9 100 alone (integer ALU and multiply-add pipes together; latency alone).  FP64 sweeps: M = 1000, 3 free
+// parameters, 120 -> 42 us; M = 32768, 7 free, 341 -> 97 us.  Of these the formats that follow a gate's range and the
+// FP64 additions cost 2 %, and the Jacobians' normalised products 7 % of an FP64 leapfrog step (M = 16384: 2435 ->
+// 2607 us for four trajectories of 20 steps).  Normals by the FP64 functions: some 90 FP64 instructions each; here 350
+// cycles.
 //
 // Integer arithmetic gives the same bits in every kernel and on the host, so the file also compiles as plain C++.
 #pragma once
@@ -74,6 +80,26 @@ template <bool kCentred = false> PIMC_HD int64_t fx_smul(int64_t a, int64_t b)
     const int32_t a0 = (int32_t)((uint32_t)a >> 1), b0 = (int32_t)((uint32_t)b >> 1);
     const int64_t t = (int64_t)a1 * b0 + (int64_t)a0 * b1 + (kCentred ? 2684354560ll : 0ll);  // 1.25 2^31
     return (int64_t)a1 * b1 + (t >> 31);
+#endif
+}
+
+// a b / 2^(64 - kMore) to the nearest: kMore more result bits, where the product leaves room for them, and the low halves'
+// product counted.  Left out is the lowest bit of each operand times the other's high half: below half a unit of fx_smul,
+// nothing for even operands and little for small ones.
+template <int kMore> PIMC_HD int64_t fx_smul_more(int64_t a, int64_t b)
+{
+    const int32_t a1 = (int32_t)(a >> 32), b1 = (int32_t)(b >> 32);
+    const int32_t a0 = (int32_t)((uint32_t)a >> 1), b0 = (int32_t)((uint32_t)b >> 1);
+    constexpr int64_t half = 1ll << (30 - kMore);
+#ifdef __CUDA_ARCH__
+    int64_t t = (int64_t)(__umulhi((uint32_t)a, (uint32_t)b) >> 1) + half, r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(a1), "r"(b0), "l"(t));
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(a0), "r"(b1), "l"(t));
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a1), "r"(b1));
+    return (int64_t)((uint64_t)r << kMore) + (t >> (31 - kMore));
+#else
+    const int64_t t = (int64_t)a1 * b0 + (int64_t)a0 * b1 + (int64_t)(((uint64_t)(uint32_t)a * (uint32_t)b) >> 33) + half;
+    return (int64_t)((uint64_t)((int64_t)a1 * b1) << kMore) + (t >> (31 - kMore));
 #endif
 }
 
@@ -202,6 +228,32 @@ PIMC_HD double fx_double(int64_t a, int f)
     const uint64_t r = ((uint64_t)(1085 - lz - f) << 52) + (m >> 11) + ((m >> 10) & 1ull);
     return fx_from_bits(r | ((uint64_t)a & 0x8000000000000000ull));
 }
+
+// ---- normalised values ----------------------------------------------------------------------------------------------
+
+// A signed value with its exponent taken out, m 2^-f, for products that keep their relative precision however small the
+// factors are: 2^62 <= |m| < 2^63 from fx_norm and fx_norm_of, a bit less with every product.
+struct Fxn {
+    int64_t m;
+    int f;
+};
+// v in format f (values below 2^31 keep leading zeros).
+PIMC_HD Fxn fx_norm(int64_t v, int f)
+{
+    const uint32_t h = (uint32_t)((uint64_t)(v < 0 ? -v : v) >> 32);
+    const int lz = fx_clz32(h | 1u) - 1;
+    return {(int64_t)fx_shl((uint64_t)v, lz), f + lz};
+}
+// From a double (zero for a subnormal one).
+PIMC_HD Fxn fx_norm_of(double v)
+{
+    const uint64_t b = fx_bits(v);
+    const int ex = (int)((b >> 52) & 0x7ffu);
+    const int64_t m = ex ? (int64_t)(((b & 0xfffffffffffffull) | 0x10000000000000ull) << 10) : 0;
+    return {(b >> 63) ? -m : m, 1085 - ex};
+}
+PIMC_HD Fxn fx_fmul(const Fxn& a, const Fxn& b) { return {fx_smul<true>(a.m, b.m) * 2, a.f + b.f - 63}; }
+PIMC_HD double fx_double(const Fxn& a) { return fx_double(a.m, a.f); }
 
 // ---- 2^-y, 1/d -------------------------------------------------------------------------------------------------------
 
@@ -338,14 +390,14 @@ PIMC_HD int64_t fx_recip(uint64_t mag, int& lz)
     const int32_t e43 = (int32_t)(e >> 19);
     const int64_t w = e + (((int64_t)e43 * e43) >> 24);
     const int64_t x1 = (int64_t)x0 << 31;  // format 61
-    return x1 + (fx_smul(x1, w * (1 << 20)) >> 18);
+    return x1 + (fx_smul(x1, (int64_t)((uint64_t)w << 20)) >> 18);
 }
 
 // ---- the HH map ------------------------------------------------------------------------------------------------------
 
 // Constants of the step dt (host-made, passed to the kernels by value).  ok: dt lies in the range of the formats.
 struct HhFixed {
-    int64_t c_bn, c_ah, c_bm;  // format 61: dt beta_n, dt alpha_h, dt beta_m at V = -101
+    int64_t c_bn, c_ah, c_bm;  // dt beta_n (format 67), dt alpha_h (68), dt beta_m (62) at V = -101
     int64_t dt67, dt10, dt100; // dt (67), dt/10 (70), dt/100 (73)
     int ok;
 };
@@ -355,9 +407,9 @@ inline HhFixed hh_fixed_of(double dt)
     HhFixed c{};
     c.ok = dt >= 0.01 && dt <= 0.04;
     if (!c.ok) return c;
-    c.c_bn = fx_of(dt * 0.1960390231862711014, 61);  // 0.125 e^{36/80}
-    c.c_ah = fx_of(dt * 0.42347532250890622586, 61); // 0.07 e^{36/20}
-    c.c_bm = fx_of(dt * 29.556224395722600909, 61);  // 4 e^{36/18}
+    c.c_bn = fx_of(dt * 0.1960390231862711014, 67);  // 0.125 e^{36/80}
+    c.c_ah = fx_of(dt * 0.42347532250890622586, 68); // 0.07 e^{36/20}
+    c.c_bm = fx_of(dt * 29.556224395722600909, 62);  // 4 e^{36/18}
     c.dt67 = fx_of(dt, 67);
     c.dt10 = fx_of(dt / 10.0, 70);
     c.dt100 = fx_of(dt / 100.0, 73);
@@ -367,6 +419,7 @@ inline HhFixed hh_fixed_of(double dt)
 // Model parameters in fixed point: conductances, reversal potentials, kappa = dt/C.
 struct HhFixedParams {
     int64_t gNa, gK, gL, ENa, EK, EL, kappa;  // formats 55, 57, 60, 55, 55, 55, 66
+    Fxn kap;                                  // kappa without the rounding of dt (1/C)
     bool ok;
 };
 
@@ -384,6 +437,7 @@ PIMC_HD HhFixedParams hh_fixed_params(const HhFixed& c, const double* q, double 
     p.EK = fx_of(q[4], 55);
     p.EL = fx_of(q[5], 55);
     p.kappa = fx_of(kappa, 66);
+    p.kap = fx_fmul(fx_norm_of(dt), fx_norm_of(q[7]));
     return p;
 }
 
@@ -410,162 +464,171 @@ PIMC_HD int64_t fx_dpsi_series(int64_t v)
     return (kFxOne62 >> 1) + (fx_smul(fx_smul(u, s3), 0xaaaaaaaaaaaaaabll) * 2);  // u s3: format 63; /6 (1/6, 62): 61
 }
 
-// psi'(u) for |u| >= 1/16 in format 62, from v = 10 u (55), p = 10 psi (52), x and s with 1/|1 - e^{-u}| = x 2^s.
+// psi'(u) for |u| >= 1/16 in format 62, from v = 10 u (55), p = 10 psi (55), x and s with 1/|1 - e^{-u}| = x 2^s.
 PIMC_HD int64_t fx_dpsi(int64_t v, int64_t p, int64_t x, int s)
 {
     const int64_t u = fx_smul(v, 0x6666666666666666ll);                              // format 57
-    const int64_t psi = fx_smul((int64_t)((uint64_t)p << 3), 0x6666666666666666ll);  // format 57
+    const int64_t psi = fx_smul(p, 0x6666666666666666ll);  // format 57
     int64_t n = ((int64_t)1 << 57) + u - psi;  // the sign of 1 - e^{-u}
     n = n < 0 ? -n : n;
     const int64_t q = fx_smul((int64_t)fx_shl((uint64_t)n << 3, s > 0 ? s & 15 : 0), x);  // format 57
     return fx_sar(q, s < 0 ? -s & 31 : 0) * 32;
 }
 
-// Gate rates at V (format 55, |V| < 100): a[g] = dt alpha, l[g] = dt (alpha + beta) of m, h, n in format 60.  With
-// t = V + 101 in (1, 201): e^{-t/80} and e^{-t/18} from the table, e^{-t/20} and B = e^{-t/10} by squaring mantissas;
-// 1 - e^{-u} of alpha_m and alpha_n and 1 + e^{-(V+35)/10} of beta_h from B scaled by 2^-k, which keeps all three
-// below 1 at every V.
-// With kAdj also d[g] = dt d(alpha)/dV and e[g] = dt d(beta)/dV (format 60):
-// alpha' from psi'(u) = (1 + u - psi)/(1 - e^{-u}), or its series.
+// Gate rates at V (format 55, |V| < 100), each gate's in a format of its own, as fine as its range allows (the small
+// values of a gate are rounded finely in FP64, too): a[g] = dt alpha in formats 62 (m), 67 (h), 64 (n), l[g] =
+// dt (alpha + beta) in 62, 67, 66.  With t = V + 101 in (1, 201): e^{-t/80} and e^{-t/18} from the table, e^{-t/20} and
+// B = e^{-t/10} by squaring mantissas; 1 - e^{-u} of alpha_m and alpha_n and 1 + e^{-(V+35)/10} of beta_h from B scaled
+// by 2^-k, which keeps all three below 1 at every V.
+// With kAdj also da[g] = dt d(alpha)/dV and db[g] = dt d(beta)/dV in formats fd[g]: 66 (m), 70 to 78 (h, whose
+// derivatives fall with V), 71 (n); alpha' from psi'(u) = (1 + u - psi)/(1 - e^{-u}), or its series.
 template <bool kAdj>
-PIMC_HD void hh_fixed_rates(const HhFixed& c, int64_t V, int64_t a[3], int64_t l[3], int64_t* da, int64_t* db)
+PIMC_HD void hh_fixed_rates(const HhFixed& c, int64_t V, int64_t a[3], int64_t l[3], int64_t* da, int64_t* db, int* fd)
 {
     const uint64_t U = ((uint64_t)V + (101ull << 55)) << 1;                   // t, format 56
     const uint64_t z80 = 0ull - fx_umul(U, 0x93bb62877cdff3c9ull);           // -t log2(e)/80, format 61, modulo 8
     const uint64_t z18 = 0ull - fx_umul(U, 0xa42589ebe01547c3ull);           // -t log2(e)/18, format 59, modulo 32
     const uint64_t m1 = fx_exp2_mant(z80 << 3), m18 = fx_exp2_mant(z18 << 5);
-    const int e1 = (int)(z80 >> 61) - 8, e18 = (int)(z18 >> 59) - 32;
+    const int e1 = (int)(z80 >> 61) - 8, e18 = (int)(z18 >> 59) - 32;         // both negative
     int e4 = e1;
     const uint64_t m4 = fx_square(fx_square(m1, e4), e4);
     int e8 = e4;
     const uint64_t m8 = fx_square(m4, e8);                                    // B = m8 2^e8, -30 < e8 <= 0
 
-    const int64_t bn = fx_sar((int64_t)fx_umul(m1, (uint64_t)c.c_bn), -e1);    // dt beta_n, format 60
-    const int64_t ah = fx_sar((int64_t)fx_umul(m4, (uint64_t)c.c_ah), -e4);    // dt alpha_h
-    const int64_t bm = fx_sar((int64_t)fx_umul(m18, (uint64_t)c.c_bm), -e18);  // dt beta_m
+    const int64_t bn = fx_sar((int64_t)fx_umul(m1, (uint64_t)c.c_bn), -e1);        // dt beta_n, format 66
+    const int64_t ah4 = (int64_t)fx_umul(m4, (uint64_t)c.c_ah), ah = fx_sar(ah4, -e4);  // dt alpha_h, format 67
+    const int64_t bm = fx_sar((int64_t)fx_umul(m18, (uint64_t)c.c_bm), -e18 - 1);  // dt beta_m, format 62
 
     // e^{6.1} = 1.7416 2^8, e^{4.6} = 1.5544 2^6, e^{6.6} = 1.4357 2^9: e^{-u_m}, e^{-u_n}, e^{-(V+35)/10} over B
     const int k = 11 + e8 > 0 ? 11 + e8 : 0, b = -e8 - 11 + k;  // b = max(0, -e8 - 11)
     const int64_t one = (int64_t)((uint64_t)((uint32_t)(kFxOne62 >> 32) >> k) << 32);
     const int64_t Dm = one - fx_sar((int64_t)(fx_umul(m8, 0xdeedcb68f9f2df6dull) >> 1), 2 + b);
     const int64_t Dn = one - fx_sar((int64_t)(fx_umul(m8, 0xc6f7f83846180a73ull) >> 1), 4 + b);
-    const int64_t Dh = one + fx_sar((int64_t)(fx_umul(m8, 0xb7c617949e4d1866ull) >> 1), 1 + b);
+    const int64_t Eh = (int64_t)(fx_umul(m8, 0xb7c617949e4d1866ull) >> 1), Dh = one + fx_sar(Eh, 1 + b);
     int zm, zn, zh;
     const int64_t xm = fx_recip((uint64_t)(Dm < 0 ? -Dm : Dm), zm);
     const int64_t xn = fx_recip((uint64_t)(Dn < 0 ? -Dn : Dn), zn);
     const int64_t xh = fx_recip((uint64_t)Dh, zh);
     // 10 u/(1 - e^{-u}) = (V + V0) x 2^s, s = z - 2 - k: a left shift goes before the product (it comes with a small
-    // V + V0), a right shift after it.  u and 1 - e^{-u} have the same sign.
+    // V + V0), a right shift after it.  u and 1 - e^{-u} have the same sign.  beta_h = x 2^-s with s >= 1.
     const int64_t vm = V + (40ll << 55), vn = V + (55ll << 55);
     const int sm = zm - 2 - k, sn = zn - 2 - k, shh = k + 2 - zh;
-    const int64_t pm = fx_sar(fx_smul<true>((int64_t)fx_shl((uint64_t)(vm < 0 ? -vm : vm), sm > 0 ? sm & 15 : 0), xm),
-                              sm < 0 ? -sm & 31 : 0);
+    const int64_t pm = fx_sar(fx_smul_more<3>((int64_t)fx_shl((uint64_t)(vm < 0 ? -vm : vm), sm > 0 ? sm & 15 : 0), xm),
+                              sm < 0 ? -sm & 31 : 0);  // below 160: format 55
     const int64_t pn = fx_sar(fx_smul<true>((int64_t)fx_shl((uint64_t)(vn < 0 ? -vn : vn), sn > 0 ? sn & 15 : 0), xn),
-                              sn < 0 ? -sn & 31 : 0);
-    int64_t am = fx_smul<true>(pm, c.dt10) << 2, an = fx_smul<true>(pn, c.dt100) >> 1;
-    const int64_t bh = fx_sar(fx_smul(c.dt67, xh), 4 + shh);
+                              sn < 0 ? -sn & 31 : 0) * 8;  // its 2^-52 is 2^-64 in dt alpha_n
+    int64_t am = fx_smul_more<1>(pm, c.dt10), an = fx_smul<true>(pn, c.dt100);
+    const int64_t bx = fx_smul(c.dt67, xh) << 2, bh = fx_sar(bx, shh - 1);
     // |u| < 1/16: the series (the quotient above is not used there)
     constexpr int64_t kCut = 5ll << 52;  // 10/16, format 55
     const bool cut_m = fx_inside(vm, kCut), cut_n = fx_inside(vn, kCut);
-    if (cut_m) am = fx_smul(c.dt67, fx_psi_series(vm)) >> 5;
-    if (cut_n) an = fx_smul(c.dt10, fx_psi_series(vn)) >> 8;
+    if (cut_m) am = fx_smul(c.dt67, fx_psi_series(vm)) >> 3;
+    if (cut_n) an = fx_smul(c.dt10, fx_psi_series(vn)) >> 4;
     if (kAdj) {
         const int64_t dm = cut_m ? fx_dpsi_series(vm) : fx_dpsi(vm, pm, xm, sm);
         const int64_t dn = cut_n ? fx_dpsi_series(vn) : fx_dpsi(vn, pn, xn, sn);
-        da[0] = fx_smul(c.dt10, dm) >> 8;
-        da[1] = fx_smul(ah, -0x666666666666666ll) * 2;                         // -alpha_h/20 (-0.1 in format 62, halved)
-        da[2] = fx_smul(c.dt100, dn) >> 11;
-        db[0] = -fx_smul(bm * 4, 0x38e38e38e38e38ell);                         // -beta_m/18 (1/18 in format 62)
-        const int64_t b61 = fx_sar(xh, shh);                                   // beta_h, format 61
-        db[1] = fx_smul(fx_smul(bh, ((int64_t)1 << 62) - b61 * 2), 0x6666666666666666ll);  // beta_h (1 - beta_h)/10
-        db[2] = -fx_smul(bn * 4, 0xcccccccccccccdll);                          // -beta_n/80 (1/80 in format 62)
+        da[0] = fx_smul(c.dt10, dm) >> 2;
+        db[0] = fx_smul(bm, -0x71c71c71c71c71c7ll) * 2;                        // -beta_m/18 (8/18 of 2^64)
+        // -alpha_h/20 (8/20 of 2^64) and beta_h (1 - beta_h)/10 = beta_h^2 e^{-(V+35)/10}/10 (4/10 of 2^64)
+        const int x = -e4 - 4 < 0 ? 0 : (-e4 - 4 > 8 ? 8 : -e4 - 4);
+        da[1] = fx_sar(fx_smul(ah4, -0x6666666666666666ll), -e4 - x);
+        const int64_t bb = fx_smul(fx_smul(bx, fx_smul(Eh, xh) << 2), 0x6666666666666666ll);
+        const int r = b + 2 * shh - k - x, r1 = r > 0 ? 1 : 0;                 // 0 to 12; bb below 2^59.6, below 2^59 at r = 0
+        db[1] = fx_sar(bb << (4 - r1), r - r1);
+        da[2] = fx_smul(c.dt100, dn);
+        db[2] = fx_smul(bn, -0x6666666666666666ll);                            // -beta_n/80 (32/80 of 2^64)
+        fd[0] = 66;
+        fd[1] = 70 + x;
+        fd[2] = 71;
     }
     a[0] = am;
     a[1] = ah;
     a[2] = an;
     l[0] = am + bm;
     l[1] = ah + bh;
-    l[2] = an + bn;
+    l[2] = (an << 2) + bn;
 }
 
-// The part of a stage that no parameter enters: the gates' increments dt F (format 59) in k[0..2], m^3 h and n^4 (format
+// The increments dt F of the gates at state s (format 62) from the rates: formats 62 (m), 66 (h), 64 (n).  The products'
+// errors are a quarter of a unit of 2^-60 (m), 2^-65 (h), 2^-64 (n).
+PIMC_HD void hh_fixed_increments(const int64_t a[3], const int64_t l[3], const int64_t* s, int64_t* k)
+{
+    k[0] = a[0] - fx_smul_more<2>(l[0], s[0]);
+    k[1] = (a[1] >> 1) - fx_smul_more<1>(l[1], s[1]);
+    k[2] = a[2] - fx_smul<true>(l[2], s[2]);
+}
+
+// The part of a stage that no parameter enters: the gates' increments in k[0..2], m^3 h and n^4 (format
 // 60) in k[3], k[4].  A site's parameter moves share the first stage's (the path stands still during them).
 PIMC_HD void hh_fixed_gates(const HhFixed& c, int64_t V, const int64_t* s, int64_t* k)
 {
     int64_t a[3], l[3];
-    hh_fixed_rates<false>(c, V, a, l, nullptr, nullptr);
-#pragma unroll
-    for (int g = 0; g < 3; ++g) k[g] = (a[g] >> 1) - fx_smul<true>(l[g] * 4, s[g]);
-    const int64_t m = s[0] * 2, h = s[1] * 2, n = s[2] * 2;  // format 62
-    const int64_t m2 = fx_smul(m, m) * 4, mh = fx_smul(m, h) * 4, n2 = fx_smul(n, n) * 4;
+    hh_fixed_rates<false>(c, V, a, l, nullptr, nullptr, nullptr);
+    hh_fixed_increments(a, l, s, k);
+    const int64_t m2 = fx_smul(s[0], s[0]) * 4, mh = fx_smul(s[0], s[1]) * 4, n2 = fx_smul(s[2], s[2]) * 4;  // format 62
     k[3] = fx_smul<true>(m2, mh);
     k[4] = fx_smul<true>(n2, n2);
 }
 
-// The increment of V, K[0] (format 50), from m^3 h and n^4; false when a term leaves its format.
-PIMC_HD bool hh_fixed_current(const HhFixedParams& p, int64_t I45, int64_t V, int64_t m3h, int64_t n4, int64_t* K)
+// The increment of V, K[0] (format 51), from m^3 h and n^4; false when a term or a gate's increment K[1..3] leaves its
+// format.
+PIMC_HD bool hh_fixed_current(const HhFixedParams& p, int64_t I46, int64_t V, int64_t m3h, int64_t n4, int64_t* K)
 {
     const int64_t tNa = fx_smul<true>(V - p.ENa, (int64_t)((uint64_t)m3h << 2));    // format 53
     const int64_t tK = fx_smul<true>(V - p.EK, (int64_t)((uint64_t)n4 << 2));
-    constexpr int64_t kTwo = 1ll << 61, kT = 1ll << 61, kS = 1ll << 59;       // 2, 256, 2^14
-    const bool ok = fx_inside(m3h, kTwo) && fx_inside(n4, kTwo) && fx_inside(tNa, kT) && fx_inside(tK, kT);
-    const int64_t S = I45 - fx_smul<true>(p.gNa, (int64_t)((uint64_t)tNa << 1)) -
-                      (fx_smul<true>(p.gK, (int64_t)((uint64_t)tK << 1)) >> 2) - (fx_smul<true>(p.gL, V - p.EL) >> 6);
-    K[0] = fx_smul<true>((int64_t)((uint64_t)S << 3), p.kappa);
-    constexpr int64_t kK = 100ll << 50;
+    constexpr int64_t kTwo = 1ll << 61, kT = 1ll << 61, kS = 1ll << 60;       // 2, 256, 2^14
+    constexpr int64_t kM = 0x27ae147a00000000ll, kH = 0x2aaaaaaa00000000ll;  // 0.62 (62), 1/24 (66)
+    const bool ok = fx_inside(m3h, kTwo) && fx_inside(n4, kTwo) && fx_inside(tNa, kT) && fx_inside(tK, kT) &&
+                    fx_inside(K[1], kM) && fx_inside(K[2], kH);
+    const int64_t tKL = fx_smul<true>(p.gK, (int64_t)((uint64_t)tK << 2)) + (fx_smul<true>(p.gL, V - p.EL) >> 3);  // 48
+    const int64_t S = I46 - fx_smul<true>(p.gNa, (int64_t)((uint64_t)tNa << 2)) - ((tKL + 2) >> 2);
+    K[0] = fx_smul_more<1>((int64_t)((uint64_t)S << 2), p.kappa);
+    constexpr int64_t kK = 100ll << 51;
     return ok && fx_inside(S, kS) && fx_inside(K[0], kK);
 }
 
-// What the reverse pass of one stage takes: the Jacobian of its increments K = dt F, as doubles.
-//   kJlam: -dK_g/ds_g (3), kJgam: dK_g/dV (3), kJV: dK_0/dV, kJg: dK_0/ds_g (3), and -dK_0/dgNa, -dK_0/dgK, -dK_0/dgL,
+// What the reverse pass of one stage takes: the Jacobian of its increments K = dt F, as doubles of FP64's own relative
+// precision (the small entries below threshold -- m^3 h is 1e-4 there -- are what data without spikes have):
+//   kJlam: -dK_g/ds_g (3), kJgam: dK_g/dV (3), kJV: dK_0/dV, kJg: -dK_0/ds_g (3), and -dK_0/dgNa, -dK_0/dgK, -dK_0/dgL,
 //   dK_0/dENa, dK_0/dEK, K_0 (dK_0/dEL = kappa gL and dK_0/dC = -K_0/C are the caller's).
 enum { kJlam = 0, kJgam = 3, kJV = 6, kJg = 7, kJp = 10, kJlen = 16 };
 
-// A stage's increments -- K[0] of V (format 50), K[1..3] of the gates (format 59) -- and its Jacobian: element j goes to J[j * stride].
-PIMC_HD bool hh_fixed_stage_adj(const HhFixed& c, const HhFixedParams& p, int64_t I45, int64_t V, const int64_t* s,
-                                int64_t* K, double* J, int stride)
+// A stage's increments -- K[0] of V (format 51), K[1..3] of the gates (as hh_fixed_increments) -- and its Jacobian:
+// element j goes to J[j * stride].  sn: the gates s normalised; kNa, kK: kappa gNa, kappa gK; kq: kappa I, gNa, gK, gL
+// and kappa gL as doubles.  dK_0/dV and K_0 are sums of entries formed in FP64, whose pipe is idle here (five operations).
+PIMC_HD bool hh_fixed_stage_adj(const HhFixed& c, const HhFixedParams& p, int64_t I46, int64_t V, const int64_t* s,
+                                const Fxn* sn, const Fxn& kNa, const Fxn& kK, const double* kq, int64_t* K, double* J,
+                                int stride)
 {
     int64_t a[3], l[3], da[3], db[3];
-    hh_fixed_rates<true>(c, V, a, l, da, db);
+    int fd[3];
+    hh_fixed_rates<true>(c, V, a, l, da, db, fd);
+    hh_fixed_increments(a, l, s, K + 1);
+    constexpr int kFl[3] = {62, 67, 66};
 #pragma unroll
     for (int g = 0; g < 3; ++g) {
-        K[1 + g] = (a[g] >> 1) - fx_smul<true>(l[g] * 4, s[g]);
-        J[(kJlam + g) * stride] = fx_double(l[g], 60);
-        J[(kJgam + g) * stride] = fx_double(da[g] - fx_smul((da[g] + db[g]) * 4, s[g]) * 2, 60);
+        J[(kJlam + g) * stride] = fx_double(l[g], kFl[g]);
+        J[(kJgam + g) * stride] = fx_double(da[g] - fx_smul_more<2>(da[g] + db[g], s[g]), fd[g]);
     }
-    const int64_t m = s[0] * 2, h = s[1] * 2, n = s[2] * 2;  // format 62
-    const int64_t m2 = fx_smul(m, m) * 4, mh = fx_smul(m, h) * 4, n2 = fx_smul(n, n) * 4;
-    const int64_t m3h = fx_smul<true>(m2, mh), n4 = fx_smul<true>(n2, n2);  // format 60
-    const int64_t m3h62 = (int64_t)((uint64_t)m3h << 2), n462 = (int64_t)((uint64_t)n4 << 2);
-    const int64_t vNa = V - p.ENa, vK = V - p.EK, vL = V - p.EL;
-    const int64_t tNa = fx_smul<true>(vNa, m3h62), tK = fx_smul<true>(vK, n462);  // format 53
-    constexpr int64_t kTwo = 1ll << 61, kT = 1ll << 61, kS = 1ll << 59, kG = 1ll << 62;
-    const int64_t kgNa57 = fx_smul(p.kappa, p.gNa), kgK59 = fx_smul(p.kappa, p.gK);  // kappa g: formats 57, 59
-    bool ok = fx_inside(m3h, kTwo) && fx_inside(n4, kTwo) && fx_inside(tNa, kT) && fx_inside(tK, kT) &&
-              fx_inside(kgNa57, kG >> 2) && fx_inside(kgK59, kG);  // kappa g below 8
-    const int64_t tNa54 = (int64_t)((uint64_t)tNa << 1), tK54 = (int64_t)((uint64_t)tK << 1);
-    const int64_t S = I45 - fx_smul<true>(p.gNa, tNa54) - (fx_smul<true>(p.gK, tK54) >> 2) - (fx_smul<true>(p.gL, vL) >> 6);
-    K[0] = fx_smul<true>((int64_t)((uint64_t)S << 3), p.kappa);
-    constexpr int64_t kK = 100ll << 50;
-    ok = ok && fx_inside(S, kS) && fx_inside(K[0], kK);
-    const int64_t kgNa = (int64_t)((uint64_t)kgNa57 << 3), kgK = (int64_t)((uint64_t)kgK59 << 1);  // format 60
-    const int64_t g1 = fx_smul(kgNa, m3h62) >> 1, g2 = fx_smul(kgK, n462) >> 1;                    // format 57
-    const int64_t g3 = fx_smul(p.kappa, p.gL) >> 5;                                                // format 57
-    J[kJV * stride] = fx_double(-(g1 + g2 + g3), 57);
-    // m^2 h, m^3 and n^3 in format 60 (below 4), times V - E: format 52, below 512 and so format 54; kappa g times that:
-    // format 50 (n: 4 times it, format 48)
-    const int64_t m2h = fx_smul(m2, h), m3 = fx_smul(m2, m), n3 = fx_smul(n2, n);
-    const int64_t tm = fx_smul(vNa, m2h * 2), th = fx_smul(vNa, m3 * 2), tn = fx_smul(vK, n3 * 2);
-    ok = ok && fx_inside(tm, kTwo) && fx_inside(th, kTwo) && fx_inside(tn, kTwo);
-    J[(kJg + 0) * stride] = fx_double(-3 * fx_smul(kgNa, (int64_t)((uint64_t)tm << 2)), 50);
-    J[(kJg + 1) * stride] = fx_double(-fx_smul(kgNa, (int64_t)((uint64_t)th << 2)), 50);
-    J[(kJg + 2) * stride] = fx_double(-fx_smul(kgK, (int64_t)((uint64_t)tn << 2)), 48);
-    J[(kJp + 0) * stride] = fx_double(fx_smul(p.kappa, tNa54), 56);
-    J[(kJp + 1) * stride] = fx_double(fx_smul(p.kappa, tK54), 56);
-    J[(kJp + 2) * stride] = fx_double(fx_smul(p.kappa, vL), 57);
-    J[(kJp + 3) * stride] = fx_double(g1, 57);
-    J[(kJp + 4) * stride] = fx_double(g2, 57);
-    J[(kJp + 5) * stride] = fx_double(K[0], 50);
+    const int64_t m2 = fx_smul(s[0], s[0]) * 4, mh = fx_smul(s[0], s[1]) * 4, n2 = fx_smul(s[2], s[2]) * 4;  // format 62
+    const bool ok = hh_fixed_current(p, I46, V, fx_smul<true>(m2, mh), fx_smul<true>(n2, n2), K);
+    const Fxn vNa = fx_norm(V - p.ENa, 55), vK = fx_norm(V - p.EK, 55), vL = {V - p.EL, 55};
+    const Fxn mm = fx_fmul(sn[0], sn[0]), m3 = fx_fmul(mm, sn[0]), vmm = fx_fmul(vNa, mm), vm3 = fx_fmul(vmm, sn[0]);
+    const Fxn nn = fx_fmul(sn[2], sn[2]), n3 = fx_fmul(nn, sn[2]), vn3 = fx_fmul(vK, n3);
+    const Fxn gm = fx_fmul(kNa, fx_fmul(vmm, sn[1])), gn = fx_fmul(kK, vn3);
+    const double dNa = fx_double(fx_fmul(p.kap, fx_fmul(vm3, sn[1]))), dK = fx_double(fx_fmul(p.kap, fx_fmul(vn3, sn[2])));
+    const double dL = fx_double(fx_fmul(p.kap, vL));
+    const double eNa = fx_double(fx_fmul(kNa, fx_fmul(m3, sn[1]))), eK = fx_double(fx_fmul(kK, fx_fmul(n3, sn[2])));
+    J[(kJg + 0) * stride] = fx_double((gm.m >> 2) * 3, gm.f - 2);
+    J[(kJg + 1) * stride] = fx_double(fx_fmul(kNa, vm3));
+    J[(kJg + 2) * stride] = fx_double(gn.m, gn.f - 2);
+    J[(kJp + 0) * stride] = dNa;
+    J[(kJp + 1) * stride] = dK;
+    J[(kJp + 2) * stride] = dL;
+    J[(kJp + 3) * stride] = eNa;
+    J[(kJp + 4) * stride] = eK;
+    J[(kJp + 5) * stride] = fma(-kq[3], dL, fma(-kq[2], dK, fma(-kq[1], dNa, kq[0])));
+    J[kJV * stride] = -(eNa + eK + kq[4]);
     return ok;
 }
 
@@ -573,8 +636,34 @@ PIMC_HD bool hh_fixed_stage_adj(const HhFixed& c, const HhFixedParams& p, int64_
 // below 2; sampled gates scatter past 1 at the spikes).
 PIMC_HD bool hh_fixed_inside(int64_t V, const int64_t* s)
 {
-    constexpr int64_t kV = 100ll << 55, kS = 0x2d1eb85100000000ll;  // 1.41, format 61
+    constexpr int64_t kV = 100ll << 55, kS = 0x5a3d70a300000000ll;  // 1.41, format 62
     return fx_inside(V, kV) && fx_inside(s[0], kS) && fx_inside(s[1], kS) && fx_inside(s[2], kS);
+}
+
+// The next stage's state and the weighted sums of the increments after stage st (weights 1, 2, 2, 1): aV in format 51,
+// as[g] in formats 61 (m), 65 (h), 63 (n): room for six increments, below 0.62, 1/24 (both checked) and 0.153.
+PIMC_HD void hh_fixed_step(int st, int64_t V0, const int64_t* s0, const int64_t* K, int64_t& V, int64_t* s, int64_t& aV,
+                           int64_t* as)
+{
+    const int w = (st == 1 || st == 2) ? 1 : 0, d = st < 2 ? 0 : 1;  // weight 2^w; next stage at x + K 2^(d - 1)
+    constexpr int kTo62[3] = {1, 5, 3};                              // K[1 + g] / 2 to format 62
+    aV += K[0] << w;
+    V = V0 + (K[0] << (3 + d));
+#pragma unroll
+    for (int g = 0; g < 3; ++g) {
+        as[g] += w ? K[1 + g] : (K[1 + g] + (st >> 1)) >> 1;  // one rounding down, one up
+        s[g] = s0[g] + (K[1 + g] >> (kTo62[g] - d));
+    }
+}
+
+// f from the sums.  The gates' increment is added to x in FP64: rounded once, with every bit of a small x in it.
+PIMC_HD void hh_fixed_result(const double* x, int64_t V0, int64_t aV, const int64_t* as, double* f)
+{
+    constexpr int64_t kSixth = 0x5555555555555555ll;  // 1/6, format 65
+    f[0] = fx_double(V0 + fx_smul<true>(aV * 4, kSixth) * 2, 55);
+    f[1] = x[1] + fx_double(fx_smul<true>(as[0], kSixth), 62);
+    f[2] = x[2] + fx_double(fx_smul_more<1>(as[1], kSixth), 67);
+    f[3] = x[3] + fx_double(fx_smul<true>(as[2], kSixth), 64);
 }
 
 // One RK4 step of the HH field, f = x + (K1 + 2 K2 + 2 K3 + K4)/6, drive held at I.  False (f untouched) when a value
@@ -587,16 +676,16 @@ PIMC_HD bool hh_map_fixed(const HhFixed& c, const HhFixedParams& p, const double
     if (!p.ok || !fx_below(x[0], 100.0) || !fx_below(x[1], 1.375) || !fx_below(x[2], 1.375) ||
         !fx_below(x[3], 1.375) || !fx_below(I, 16384.0))
         return false;
-    const int64_t V0 = fx_of(x[0], 55), I45 = fx_of(I, 45);
+    const int64_t V0 = fx_of(x[0], 55), I46 = (fx_of(I, 47) + 1) >> 1;
     int64_t s0[3], V = V0, s[3], aV = 0, as[3] = {0, 0, 0}, K[4];
-    for (int g = 0; g < 3; ++g) s[g] = s0[g] = fx_of(x[1 + g], 61);
+    for (int g = 0; g < 3; ++g) s[g] = s0[g] = fx_of(x[1 + g], 62);
     // one copy of the stage's code: four would not fit the instruction cache
 #pragma unroll 1
     for (int st = 0; st < 4; ++st) {
         if (first == kStage1Load && st == 0) {
 #pragma unroll
             for (int g = 0; g < 3; ++g) K[1 + g] = s1[g * stride];
-            if (!hh_fixed_current(p, I45, V, s1[3 * stride], s1[4 * stride], K)) return false;
+            if (!hh_fixed_current(p, I46, V, s1[3 * stride], s1[4 * stride], K)) return false;
         } else {
             int64_t k[5];
             hh_fixed_gates(c, V, s, k);
@@ -606,22 +695,12 @@ PIMC_HD bool hh_map_fixed(const HhFixed& c, const HhFixedParams& p, const double
             }
 #pragma unroll
             for (int g = 0; g < 3; ++g) K[1 + g] = k[g];
-            if (!hh_fixed_current(p, I45, V, k[3], k[4], K)) return false;
+            if (!hh_fixed_current(p, I46, V, k[3], k[4], K)) return false;
         }
-        const int w = (st == 1 || st == 2) ? 1 : 0, d = st < 2 ? 0 : 1;  // weight 2^w; next stage at x + K 2^(d - 1)
-        aV += K[0] << w;
-        V = V0 + (K[0] << (4 + d));
-#pragma unroll
-        for (int g = 0; g < 3; ++g) {
-            as[g] += K[1 + g] << w;
-            s[g] = s0[g] + (K[1 + g] << (1 + d));
-        }
+        hh_fixed_step(st, V0, s0, K, V, s, aV, as);
         if (st < 3 && !hh_fixed_inside(V, s)) return false;
     }
-    constexpr int64_t kSixth = 0x5555555555555555ll;  // 1/6, format 65
-    f[0] = fx_double(V0 + fx_smul<true>(aV * 8, kSixth) * 2, 55);
-#pragma unroll
-    for (int g = 0; g < 3; ++g) f[1 + g] = fx_double(s0[g] + fx_smul<true>(as[g], kSixth) * 2, 61);
+    hh_fixed_result(x, V0, aV, as, f);
     return true;
 }
 
@@ -633,26 +712,25 @@ PIMC_HD bool hh_map_fixed_adj(const HhFixed& c, const HhFixedParams& p, const do
     if (!p.ok || !fx_below(x[0], 100.0) || !fx_below(x[1], 1.375) || !fx_below(x[2], 1.375) ||
         !fx_below(x[3], 1.375) || !fx_below(I, 16384.0))
         return false;
-    const int64_t V0 = fx_of(x[0], 55), I45 = fx_of(I, 45);
+    const int64_t V0 = fx_of(x[0], 55), I46 = (fx_of(I, 47) + 1) >> 1;
     int64_t s0[3], V = V0, s[3], aV = 0, as[3] = {0, 0, 0}, K[4];
-    for (int g = 0; g < 3; ++g) s[g] = s0[g] = fx_of(x[1 + g], 61);
+    Fxn sn[3];
+    for (int g = 0; g < 3; ++g) {
+        s[g] = s0[g] = fx_of(x[1 + g], 62);
+        sn[g] = fx_norm_of(x[1 + g]);
+    }
+    const Fxn kNa = fx_fmul(p.kap, fx_norm(p.gNa, 55)), kK = fx_fmul(p.kap, fx_norm(p.gK, 57));
+    const double kq[5] = {fx_double(fx_fmul(p.kap, fx_norm_of(I))), fx_double(p.gNa, 55), fx_double(p.gK, 57),
+                          fx_double(p.gL, 60), fx_double(fx_fmul(p.kap, fx_norm(p.gL, 60)))};
 #pragma unroll 1
     for (int st = 0; st < 4; ++st) {
-        if (!hh_fixed_stage_adj(c, p, I45, V, s, K, J + (int64_t)st * kJlen * stride, stride)) return false;
-        const int w = (st == 1 || st == 2) ? 1 : 0, d = st < 2 ? 0 : 1;
-        aV += K[0] << w;
-        V = V0 + (K[0] << (4 + d));
-#pragma unroll
-        for (int g = 0; g < 3; ++g) {
-            as[g] += K[1 + g] << w;
-            s[g] = s0[g] + (K[1 + g] << (1 + d));
-        }
+        if (!hh_fixed_stage_adj(c, p, I46, V, s, sn, kNa, kK, kq, K, J + (int64_t)st * kJlen * stride, stride)) return false;
+        hh_fixed_step(st, V0, s0, K, V, s, aV, as);
         if (st < 3 && !hh_fixed_inside(V, s)) return false;
-    }
-    constexpr int64_t kSixth = 0x5555555555555555ll;
-    f[0] = fx_double(V0 + fx_smul<true>(aV * 8, kSixth) * 2, 55);
 #pragma unroll
-    for (int g = 0; g < 3; ++g) f[1 + g] = fx_double(s0[g] + fx_smul<true>(as[g], kSixth) * 2, 61);
+        for (int g = 0; g < 3; ++g) sn[g] = fx_norm(s[g], 62);
+    }
+    hh_fixed_result(x, V0, aV, as, f);
     return true;
 }
 
@@ -679,7 +757,7 @@ PIMC_HD void hh_reverse(const double* J, int stride, double kgL, double iC, cons
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
             u[0] = fma(b[1 + g], j[(kJgam + g) * stride], u[0]);
-            u[1 + g] = fma(-b[1 + g], j[(kJlam + g) * stride], b[0] * j[(kJg + g) * stride]);
+            u[1 + g] = fma(-b[1 + g], j[(kJlam + g) * stride], -b[0] * j[(kJg + g) * stride]);
         }
 #pragma unroll
         for (int a = 0; a < 4; ++a) gx[a] += u[a];

@@ -157,7 +157,7 @@ template <class Model> constexpr int adjoint_smem()
 // the stages' Jacobians by integer arithmetic, the reverse pass in FP64 with 25
 // operations a stage instead of 85 (and the forward's exponentials).  J: the
 // thread's Jacobian slots (adjoint_smem, stride kBlock); unused otherwise.
-// Measured (M = 16384, a leapfrog step): 46 -> 25 us.
+// Measured (M = 16384, a leapfrog step): 46 -> 27 us.
 template <class Model, class R>
 __device__ __forceinline__ void term_adjoint(const Ctx& c, const Coef<R>& kc, const R* wr, const R* x, const R* x1,
                                              const R* pr, R In, R In1, R* e, R* own, R* nxt, R* gp, double* J)
@@ -173,7 +173,7 @@ __device__ __forceinline__ void term_adjoint(const Ctx& c, const Coef<R>& kc, co
                     e[a] = x1[a] - f[a];
                     nxt[a] = wr[a] * e[a];
                 }
-                hh_reverse(J, kBlock, kc.dt * pr[7] * pr[2], pr[7], nxt, gx, jp);
+                hh_reverse(J, kBlock, fx_double(fx_fmul(P.kap, fx_norm_of(pr[2]))), pr[7], nxt, gx, jp);
 #pragma unroll
                 for (int a = 0; a < 4; ++a) own[a] = -gx[a];
 #pragma unroll

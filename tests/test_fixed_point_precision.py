@@ -1,0 +1,115 @@
+"""The fixed-point FP64 map and adjoint against the same formulas in FP64 arithmetic: both are compared with extended
+precision, and the fixed-point side may not be further off -- where values are small, too: below threshold m^3 h and the
+Jacobian entries made of it are 1e-4 and less, deep in a spike the gate h falls to 1e-4.  The allowances are a quarter of
+FP64's own error (two sides of one rounding differ by less over thousands of states) and, for Jacobian entries, half an
+ulp (2^-54 of the entry, one rounding)."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from .test_fixed_point import NOMINAL, L, _call_map, lib  # noqa: F401 (lib: the fixture)
+
+N = 6000
+
+
+def _steady(V):
+    a = (-(V + 40) / 10 / np.expm1(-(V + 40) / 10), 0.07 * np.exp(-(V + 65) / 20), -(V + 55) / 100 / np.expm1(-(V + 55) / 10))
+    b = (4 * np.exp(-(V + 65) / 18), 1 / (1 + np.exp(-(V + 35) / 10)), 0.125 * np.exp(-(V + 65) / 80))
+    return np.stack([x / (x + y) for x, y in zip(a, b)])
+
+
+def _psi(u):
+    small = np.abs(u) < 1e-6
+    v = np.where(small, 1, u)
+    return np.where(small, 1 + u / 2 + u * u / 12, -v / np.expm1(-v))
+
+
+def _rhs(x, q, I):  # in the arithmetic of x
+    V, m, h, n = x
+    a = (_psi((V + 40) / 10), 7 * np.exp(-(V + 65) / 20) / 100, _psi((V + 55) / 10) / 10)
+    b = (4 * np.exp(-(V + 65) / 18), 1 / (1 + np.exp(-(V + 35) / 10)), np.exp(-(V + 65) / 80) / 8)
+    dV = (I - q[0] * m ** 3 * h * (V - q[3]) - q[1] * n ** 4 * (V - q[4]) - q[2] * (V - q[5])) / q[6]
+    return np.stack([dV] + [a[g] * (1 - x[1 + g]) - b[g] * x[1 + g] for g in range(3)])
+
+
+def _map(x, q, I, dt):
+    k1 = _rhs(x, q, I)
+    k2 = _rhs(x + dt / 2 * k1, q, I)
+    k3 = _rhs(x + dt / 2 * k2, q, I)
+    k4 = _rhs(x + dt * k3, q, I)
+    return x + dt / 6 * (k1 + 2 * k2 + 2 * k3 + k4)
+
+
+def _states(kind):
+    rng = np.random.default_rng(3)
+    q = NOMINAL[:, None] * rng.uniform(0.8, 1.2, (7, N))
+    V = rng.uniform(*{"rest": (-68, -62), "spike": (-20, 40), "wide": (-78, 45), "small": (-78, 45)}[kind], N)
+    g = _steady(V)
+    if kind == "small":
+        g = 10.0 ** rng.uniform(-4, -2, (3, N))
+    elif kind == "spike":
+        g = g * rng.uniform(0.5, 1.0, (3, N))
+    elif kind == "wide":
+        g = np.minimum(g * rng.uniform(0.7, 1.3, (3, N)), 1.0)
+    x = np.concatenate([V[None], g])
+    I = rng.uniform(-5, 20, N)
+    if kind == "rest":  # net currents of 0.1
+        I = -_rhs(x, q, 0.0)[0] * q[6] + rng.uniform(-0.1, 0.1, N)
+    return x, q, I
+
+
+def _rms(v):
+    return float(np.sqrt(np.mean(np.square(v.astype(np.float64)))))
+
+
+@pytest.mark.parametrize("dt", [0.01, 0.02, 0.04])
+@pytest.mark.parametrize("kind", ["rest", "spike", "wide", "small"])
+def test_map_is_as_exact_as_fp64(lib, kind, dt):  # noqa: F811
+    x, q, I = _states(kind)
+    f, ok = _call_map(lib, dt, q, x, I)
+    ref = _map(x.astype(L), q.astype(L), I.astype(L), L(dt))
+    fp64 = _map(x, q, I, dt)
+    assert ok.mean() > 0.7  # wide states at dt = 0.04 leave the formats' range
+    e, e64 = (f - ref)[:, ok], (fp64 - ref)[:, ok]
+    assert _rms(e[0]) <= 1.25 * _rms(e64[0])
+    binade = np.floor(np.log2(np.abs(fp64[:, ok])))
+    seen = 0
+    for g in (1, 2, 3):
+        for k in range(-13, 1):
+            at = binade[g] == k
+            if at.sum() >= 200:
+                assert _rms(e[g, at]) <= 1.25 * _rms(e64[g, at]), (g, k)
+                seen += 1
+    assert seen >= 3
+
+
+@pytest.mark.parametrize("dt", [0.01, 0.02, 0.04])
+@pytest.mark.parametrize("kind", ["rest", "spike", "wide", "small"])
+def test_adjoint_is_as_exact_as_fp64(lib, kind, dt):  # noqa: F811
+    """Every entry of the Jacobian (unit cotangents) against complex steps, in extended precision and in FP64."""
+    x, q, I = _states(kind)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+    qa, xa = np.ascontiguousarray(np.concatenate([q, 1.0 / q[6:7]]).T), np.ascontiguousarray(x.T)
+    ok, got = np.zeros(N, dtype=np.uint8), np.zeros((4, 11, N))
+    for a in range(4):
+        w = np.zeros((N, 4))
+        w[:, a] = 1.0
+        f, gx, gp = np.zeros((N, 4)), np.zeros((N, 4)), np.zeros((N, 7))
+        lib.adjoint(ctypes.c_double(dt), p(qa), p(xa), p(np.ascontiguousarray(I)), p(w), ctypes.c_long(N), p(f), p(gx),
+                    p(gp), p(ok))
+        got[a, :4], got[a, 4:] = gx.T, gp.T
+    at = ok.astype(bool)
+    assert at.mean() > 0.7
+    for k in range(11):
+        col = []
+        for T, C in ((L, np.clongdouble), (np.float64, np.complex128)):
+            d = np.zeros((11, N), dtype=C)
+            d[k] = 1j * T(1e-30)
+            y = _map(x.astype(T) + d[:4], q.astype(T) + d[4:], I.astype(T), T(dt))
+            col.append(y.imag / T(1e-30))
+        for a in range(4):
+            ref = col[0][a, at]
+            scale = _rms(ref)
+            if scale > 0:
+                assert _rms(got[a, k, at] - ref) <= 1.25 * _rms(col[1][a, at] - ref) + 2.0 ** -54 * scale, (a, k)
