@@ -19,7 +19,8 @@
 // parameters, 120 -> 42 us; M = 32768, 7 free, 341 -> 97 us.  Of these the formats that follow a gate's range and the
 // FP64 additions cost 2 %, and the Jacobians' normalised products 7 % of an FP64 leapfrog step (M = 16384: 2435 ->
 // 2607 us for four trajectories of 20 steps).  Normals by the FP64 functions: some 90 FP64 instructions each; here 350
-// cycles.
+// cycles, of which the relative precision next to zeros costs 1 % of a sweep at M = 1000 (absolute formats: 5e-16 of a
+// normal's size, rms, where FP64 has 9e-17).
 //
 // Integer arithmetic gives the same bits in every kernel and on the host, so the file also compiles as plain C++.
 #pragma once
@@ -776,7 +777,8 @@ PIMC_HD void hh_reverse(const double* J, int stride, double kgL, double iC, cons
 
 // ---- draws -----------------------------------------------------------------------------------------------------------
 // The FP64 draws -- Box-Muller normals and -log u -- from their integers: the uniform (k + 1/2) 2^-52, k < 2^52, is
-// N 2^-53 with N = 2 k + 1.  Absolute errors below 2^-56, where FP64's are about 2^-53 for values near 1.
+// N 2^-53 with N = 2 k + 1.  Relative errors below 2^-53 beside the rounding, for small values as well: -log u near
+// u = 1, the radius made of it, and the sine and cosine next to their zeros are formed from normalised mantissas.
 
 // log(C_j/256), format 63, and C_j, about 256 over the middle of [1/2 + j/256, 1/2 + (j + 1)/256); C_127 = 256.
 #ifdef __CUDACC__
@@ -867,8 +869,8 @@ PIMC_HD int64_t fx_sin_table(uint32_t j)
 #endif
 }
 
-// -log(N 2^-53) for odd N < 2^53, in format F (returned): 70 for u >= 255/256, where the logarithm goes to 0, 62 for
-// other u >= 1/2, else 57.
+// -log(N 2^-53) for odd N < 2^53, in format F (returned): 57 for u < 1/2, 63 for u in [1/2, 255/256); above, where the
+// logarithm goes to 0, 70 + s with the result in [2^61, 2^62.1).
 // u = m 2^-E, m in [1/2, 1): E log 2 + log c_j - log(m c_j), with r = 1 - m c_j exact (|r| < 2^-7) and
 // -log(1 - r) = r + r^2/2 + ... + r^8/8 (error 2^-66).
 PIMC_HD int64_t fx_neglog(uint64_t N, int& F)
@@ -885,11 +887,19 @@ PIMC_HD int64_t fx_neglog(uint64_t N, int& F)
     const int64_t t4 = (kFxOne62 >> 2) + (((int64_t)r38 * t5) >> 7);       // 1/4 + ..., format 62
     const int64_t t3 = 0x1555555555555555ll + (fx_smul(r70, t4) >> 6);
     const int64_t t2 = (kFxOne62 >> 1) + (fx_smul(r70, t3) >> 6);
-    const int64_t w = r70 + (fx_smul(r70, fx_smul(r70, t2)) >> 4);         // format 70
-    const int64_t lc = fx_log_table(j);
+    const int64_t q = fx_smul(r70, t2);                                    // r/2 + r^2/3 + ..., format 68
     const int E = lz - 11;
-    F = E > 0 ? 57 : (j == 127u ? 70 : 62);
-    if (E == 0) return j == 127u ? w : (lc >> 1) + (w >> 8);
+    if (E == 0 && j == 127u) {  // r > 0: r (1 + q) from r's mantissa
+        const uint32_t rh = (uint32_t)((uint64_t)r70 >> 32);
+        const int s = (rh ? fx_clz32(rh) : 32 + fx_clz32((uint32_t)r70)) - 2;  // to [2^61, 2^62): 1 + q < 1 + 2^-8
+        const int64_t rm = (int64_t)((uint64_t)r70 << s);
+        F = 70 + s;
+        return rm + (fx_smul(rm, q << 3) >> 7);
+    }
+    const int64_t w = r70 + (fx_smul(r70, q) >> 4);                        // format 70
+    const int64_t lc = fx_log_table(j);
+    F = E > 0 ? 57 : 63;
+    if (E == 0) return lc + (w >> 7);
     // log 2 in format 57 and its rest in format 68
     return (int64_t)E * 0x162e42fefa39ef3ll + ((E * (701)) >> 11) + (lc >> 6) + (w >> 13);
 }
@@ -905,9 +915,9 @@ PIMC_HD float fx_rsqrt_seed(float d)
 #endif
 }
 
-// sqrt(2 a 2^-F) in format 59 for a > 0, 2 a 2^-F < 128 (the caller gives a = -log u at most 36.8).  With 2 a 2^-F = d 4^h, d in [1/4, 1): an FP32 seed y of
-// 1/sqrt(d) and sqrt(d) = d y (1 + e/2 + 3 e^2/8), e = 1 - d y^2 (|e| < 2^-21).
-PIMC_HD int64_t fx_sqrt2(int64_t a, int F)
+// sqrt(2 a 2^-F) for a > 0 as a mantissa in [2^61, 2^62] of format f (returned).  With 2 a 2^-F = d 4^h, d in [1/4, 1):
+// an FP32 seed y of 1/sqrt(d) and sqrt(d) = d y (1 + e/2 + 3 e^2/8), e = 1 - d y^2 (|e| < 2^-21).
+PIMC_HD int64_t fx_sqrt2(int64_t a, int F, int& f)
 {
     const uint32_t ah = (uint32_t)((uint64_t)a >> 32);
     int lz = ah ? fx_clz32(ah) : 32 + fx_clz32((uint32_t)a);
@@ -915,7 +925,7 @@ PIMC_HD int64_t fx_sqrt2(int64_t a, int F)
     int ex = 65 - F - lz;
     const int odd = ex & 1;
     const uint64_t d = ((uint64_t)a << lz) >> odd;
-    const int h = (ex + odd) >> 1;
+    f = 62 - ((ex + odd) >> 1);
     const uint32_t dh = (uint32_t)(d >> 32);
     float y = fx_rsqrt_seed((float)(dh >> 8) * 0x1p-24f);
     y = y < 1.99999988f ? y : 1.99999988f;
@@ -924,14 +934,26 @@ PIMC_HD int64_t fx_sqrt2(int64_t a, int F)
     const int64_t e = (int64_t)((1ull << 60) - fx_umul(d, (uint64_t)y0 * y0));     // format 60
     const int32_t e41 = (int32_t)(e >> 19);
     const int64_t c = (e >> 1) + ((3 * (((int64_t)e41 * e41) >> 22)) >> 3);        // format 60
-    const int64_t root = (int64_t)g + (fx_smul((int64_t)g, c * (1 << 20)) >> 16);  // format 62
-    const int sh = 3 - h;                                                          // format 59
-    return sh >= 0 ? (sh < 63 ? root >> sh : 0) : root << -sh;
+    return (int64_t)g + (fx_smul((int64_t)g, c * (1 << 20)) >> 16);                // format 62
 }
 
-// (cos, sin)(2 pi N 2^-53) in format 62: quadrant, 64 table angles a in it, and the angle difference delta
-// (|delta| <= pi/256) by its Taylor polynomials of degree 7 and 6 (errors below 2^-66 and 2^-60).
-PIMC_HD void fx_sincos(uint64_t N, int64_t& cs, int64_t& sn)
+// sin(theta) for theta = pi/2 d 2^-64 > 0, d < 2^56 (theta < 2^-7.3), as theta (1 - theta^2/6 + theta^4/120) from the mantissa
+// of d (the rest is below 2^-56 of it), in format f (returned).
+PIMC_HD int64_t fx_sin_small(uint64_t d, int& f)
+{
+    constexpr int64_t kHalfPi = 0x6487ed5110b4611all;                                       // pi/2, format 62
+    const uint32_t h = (uint32_t)(d >> 32);
+    const int s = (h ? fx_clz32(h) : 32 + fx_clz32((uint32_t)d)) - 1;
+    const int64_t t = fx_smul((int64_t)(d << 7), kHalfPi), t2 = fx_smul(t, t);              // theta (69), theta^2 (74)
+    const int64_t q = fx_smul(t2, 0xaaaaaaaaaaaaaabll - (fx_smul(t2, 0x4444444444444444ll) >> 17));  // format 72
+    const int64_t tm = fx_smul<true>((int64_t)(d << s), kHalfPi);                           // theta, format 62 + s
+    f = 62 + s;
+    return tm - (fx_smul(tm, q) >> 8);
+}
+
+// (cos, sin)(2 pi N 2^-53) in formats fc, fs (62 but next to a zero): quadrant, 64 table angles a in it, and the angle
+// difference delta (|delta| <= pi/256) by its Taylor polynomials of degree 7 and 6 (errors below 2^-66 and 2^-60).
+PIMC_HD void fx_sincos(uint64_t N, int64_t& cs, int64_t& sn, int& fc, int& fs)
 {
     const uint32_t q = (uint32_t)(N >> 51);
     const uint64_t fr = N << 13;  // fraction of the quadrant, format 64
@@ -946,11 +968,22 @@ PIMC_HD void fx_sincos(uint64_t N, int64_t& cs, int64_t& sn)
     const int32_t tc = 1431655765 - (fx_mulhi32(d42, 763549742) >> 14);                    // 1/24 - d2/720, format 35
     const int64_t c1 = fx_smul(d2, -(kFxOne62 >> 1) + (((int64_t)d42 * tc) >> 15));        // cos delta - 1, format 72
     const int64_t S = fx_sin_table(j), C = fx_sin_table(63u - j);
-    const int64_t s0 = (S >> 1) + (fx_smul(S, c1) >> 9) + (fx_smul(C, sd) >> 6);
-    const int64_t c0 = (C >> 1) + (fx_smul(C, c1) >> 9) - (fx_smul(S, sd) >> 6);
+    int64_t s0 = (S >> 1) + (fx_smul(S, c1) >> 9) + (fx_smul(C, sd) >> 6);
+    int64_t c0 = (C >> 1) + (fx_smul(C, c1) >> 9) - (fx_smul(S, sd) >> 6);
+    // within 2^-8 of a quadrant of a zero (one pair in 128)
+    const uint64_t near_end = fr >> 63 ? 0ull - fr : fr;
+    int f0 = 62;
+    if (near_end < (1ull << 56)) {
+        const int64_t z = fx_sin_small(near_end, f0);
+        if (fr >> 63) c0 = z;
+        else s0 = z;
+    }
+    const int f1 = fr >> 63 ? f0 : 62, f2 = fr >> 63 ? 62 : f0;  // of c0, s0
     const int64_t a = (q & 1u) ? -s0 : c0, b = (q & 1u) ? c0 : s0;
     cs = (q & 2u) ? -a : a;
     sn = (q & 2u) ? -b : b;
+    fc = (q & 1u) ? f2 : f1;
+    fs = (q & 1u) ? f1 : f2;
 }
 
 // N of the open-interval uniform that two Philox words give: k from the top 26 bits of each.
@@ -962,13 +995,13 @@ PIMC_HD uint64_t fx_uniform(uint32_t hi, uint32_t lo)
 // Box-Muller from four words: sqrt(-2 log u1) (cos, sin)(2 pi u2).
 PIMC_HD void fx_box_muller(uint32_t x, uint32_t y, uint32_t z, uint32_t w, double& z0, double& z1)
 {
-    int F;
+    int F, f, fc, fs;
     const int64_t L = fx_neglog(fx_uniform(x, y), F);
-    const int64_t r = fx_sqrt2(L, F);
+    const int64_t r = fx_sqrt2(L, F, f);
     int64_t c, s;
-    fx_sincos(fx_uniform(z, w), c, s);
-    z0 = fx_double(fx_smul(r, c), 57);
-    z1 = fx_double(fx_smul(r, s), 57);
+    fx_sincos(fx_uniform(z, w), c, s, fc, fs);
+    z0 = fx_double(fx_smul<true>(r, c), f + fc - 64);
+    z1 = fx_double(fx_smul<true>(r, s), f + fs - 64);
 }
 
 // -log u from two words.

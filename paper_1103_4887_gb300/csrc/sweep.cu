@@ -295,7 +295,8 @@ template <class Model, class R>
 __device__ __forceinline__ void site_draw(const Ctx& c, long long s, int64_t n, R* z, R& E)
 {
     constexpr int D = Model::D;
-#pragma unroll
+    // FP64: one copy of the fixed-point draws (M = 1000: 43.3 us a sweep, 44.4 with two)
+#pragma unroll(sizeof(R) == 8 ? 1 : 2)
     for (int pair = 0; 2 * pair < D; ++pair) {
         R z0, z1;
         const uint4 w = draw_block(c.seed, c.chain, (uint64_t)s, (uint32_t)n, kKindSite, pair);

@@ -113,3 +113,39 @@ def test_adjoint_is_as_exact_as_fp64(lib, kind, dt):  # noqa: F811
             scale = _rms(ref)
             if scale > 0:
                 assert _rms(got[a, k, at] - ref) <= 1.25 * _rms(col[1][a, at] - ref) + 2.0 ** -54 * scale, (a, k)
+
+
+@pytest.mark.parametrize("where", ["anywhere", "u near 1", "next to a zero of the sine or cosine", "both"])
+def test_draws_are_as_exact_as_fp64(lib, where):  # noqa: F811
+    """Normals and -log u relative to their own size, beside the FP64 formulas (the angle reduced exactly to its distance
+    from the nearest zero, as sincospi does); one rounding (2^-53 at most) is allowed for."""
+    rng = np.random.default_rng(17)
+    n = 20000
+    w = rng.integers(0, 1 << 32, (n, 4), dtype=np.uint64).astype(np.uint32)
+    bits = rng.integers(4, 25, n)
+    if where in ("u near 1", "both"):  # ones at the top of u1
+        w[:, 0] |= ((np.uint64(0xFFFFFFFF) << (32 - bits).astype(np.uint64)) & np.uint64(0xFFFFFFFF)).astype(np.uint32)
+    if where in ("next to a zero of the sine or cosine", "both"):  # zeros or ones below u2's quadrant bits
+        mask = (np.uint64(0x3FFFFFFF) & ~(np.uint64(0x3FFFFFFF) >> bits.astype(np.uint64))).astype(np.uint32)
+        w[:, 2] = np.where(rng.random(n) < 0.5, w[:, 2] | mask, w[:, 2] & ~mask)
+    z, e = np.zeros((n, 2)), np.zeros(n)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+    lib.draws(p(np.ascontiguousarray(w)), ctypes.c_long(n), p(z), p(e))
+    k = [((w[:, a] >> 6).astype(np.uint64) << np.uint64(26)) | (w[:, a + 1] >> 6) for a in (0, 2)]
+    got, ref = (z[:, 0], z[:, 1], e), {}
+    for T in (L, np.float64):
+        pi = 4 * np.arctan(T(1))
+        u1 = (k[0].astype(T) + T(0.5)) / T(2) ** 52
+        quad = (k[1] >> np.uint64(50)).astype(np.int64)
+        fr = ((k[1] & np.uint64((1 << 50) - 1)).astype(T) + T(0.5)) / T(2) ** 50
+        s, c = np.where(fr < 0.5, np.sin(pi / 2 * fr), np.cos(pi / 2 * (1 - fr))), \
+            np.where(fr < 0.5, np.cos(pi / 2 * fr), np.sin(pi / 2 * (1 - fr)))
+        cs = np.choose(quad, [c, -s, -c, s])
+        sn = np.choose(quad, [s, c, -s, -c])
+        E = -np.where(u1 > 0.5, np.log1p(-(T(1) - u1)), np.log(u1))
+        r = np.sqrt(2 * E)
+        ref[T] = (r * cs, r * sn, E)
+    for g, x, y in zip(got, ref[L], ref[np.float64]):
+        err, err64 = (g - x) / x, (y - x) / x
+        assert _rms(err) <= 1.25 * _rms(err64)
+        assert np.abs(err).max() <= np.abs(err64).max() + 2.0 ** -53
