@@ -273,8 +273,11 @@ template <class Model, class R> static cudaError_t refresh_t(const Ctx& c, cudaS
     refresh_cache_kernel<Model, R><<<(unsigned)((c.M + 1 + 255) / 256), 256, 0, s>>>(c);
     return cudaGetLastError();
 }
-// CTAs of the whole-path kernels: one a tile of work, at most four an SM (what
-// their registers let run at once).  A CTA's fixed FP64 work -- parameters and
+// CTAs of the whole-path kernels: one a tile of work, at most four an SM.  (Two to
+// four run at once, by their registers: FP64 HH gradient 243, action 158.  Grids of
+// just those were no faster: gradient, M = 4e4 to 3e5, 57, 66, 92, 116, 154, 209 us
+// against 59, 70, 92, 117, 150, 206; action at 1.5e5 42 against 40: whole tiles go
+// less evenly into fewer CTAs.)  A CTA's fixed FP64 work -- parameters and
 // constants into the arithmetic type, sums of its warps, some 70 instructions a
 // warp -- is then spread over many tiles (M = 10^6, FP32-mixed: action 80 ->
 // 55 us, gradient 176 -> 98 us, against up to 4096 CTAs of two tiles).

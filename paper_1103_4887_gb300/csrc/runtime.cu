@@ -211,9 +211,15 @@ constexpr int64_t kDeviceRows = 65536;
 
 // Writes one byte of every page of a pageable buffer that a copy is about to
 // fill: pages not yet mapped would be faulted in by the device, one by one
-// (512 reads of 16..130 KB: 105 -> 133 ms).
+// (512 reads of 16..130 KB: 105 -> 133 ms).  Page-locked memory is mapped, and it
+// may be the source of an upload still waiting on the stream (pimc_load_data's
+// arrays are the caller's again only after this call's synchronisation): left
+// alone.
 void touch(void* p, size_t bytes)
 {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) cudaGetLastError();
+    else if (at.type != cudaMemoryTypeUnregistered) return;
     volatile char* c = (volatile char*)p;
     for (size_t i = 0; i < bytes; i += 4096) c[i] = 0;
     if (bytes) c[bytes - 1] = 0;
