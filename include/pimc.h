@@ -329,8 +329,12 @@ int pimc_batch_sync(pimc_batch_t b);
  * slots with bounded waits (the launch is then cooperative); 1 keeps every
  * chain whole.  Without this call (or a cached choice of the autotuner), a batch
  * of fewer chains than the device holds CTAs is cut into tiles where that
- * shortens the sweep, one tile a CTA.  A chain's results do not depend on the
- * tile shape.  PIMC_ERR_ARG for values out of range. */
+ * shortens the sweep, one tile a CTA.  Such a launch starts when all its CTAs
+ * fit on the device at once, up to all that it holds, so it may wait for work of
+ * other streams and they for it; batches meant to run side by side on several
+ * streams are better kept whole (ctas_per_chain = 1; two batches of 128 chains of
+ * M = 4096 at once: 117 us a sweep cut, 91 whole; one alone 59 and 66).  A chain's
+ * results do not depend on the tile shape.  PIMC_ERR_ARG for values out of range. */
 int pimc_batch_set_tuning(pimc_batch_t b, int threads_per_cta, int ctas_per_sm, int ctas_per_chain);
 /* The current plan: CTAs of a launch, threads per CTA, chains split over
  * several CTAs (any output may be NULL). */
@@ -339,7 +343,8 @@ int pimc_batch_info(pimc_batch_t b, int* n_ctas, int* threads_per_cta, int* n_sp
  * burn-in) for each tile shape -- threads per CTA x CTAs per SM x CTAs per
  * long chain (1, 2, 4, and the plan of a batch without tuning, for which
  * *ctas_per_chain is the largest of 1, 2, 4 not above the most tiles that plan
- * gives a chain) -- and keep the fastest;
+ * gives a chain; pimc_batch_set_tuning with that number makes a plan of no more
+ * tiles than that) -- and keep the fastest;
  * the choice is cached per process for batches of the same model, precision, size and chain count. */
 int pimc_batch_autotune(pimc_batch_t b, int64_t trial_sweeps, uint64_t seed, int* threads_per_cta, int* ctas_per_sm,
                         int* ctas_per_chain);
