@@ -77,8 +77,8 @@ struct Ctx {
     int num_sms;                  // SMs of the handle's device
     HhFixed fx;                   // constants of dt of the fixed-point FP64 HH map
     double hRm, hRf[4];           // Rm / 2, Rf / 2
-    void* st1;                    // HH: first-stage values of the sites, shared by a sweep's parameter moves --
-                                  // FP64: int64 [5][ldx], FP32: float [3][ldx] -- or null
+    int64_t* st1;                 // FP64 HH, RK4: first-stage values of the sites, shared by a sweep's parameter moves
+                                  // ([5][ldx]), or null
     unsigned* chk;                // [3][ldx] site visits (even phase, odd phase, parameter-move cache
                                   // writes), then a u64 count of executed parameter moves: counted by
                                   // builds compiled with PIMC_CHECK only

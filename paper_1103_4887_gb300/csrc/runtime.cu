@@ -49,7 +49,7 @@ struct pimc_handle_s {
     DevState* st = nullptr;
     double* partials = nullptr;
     unsigned long long* halo = nullptr;   // halo packets of the resident sweep
-    void* st1 = nullptr;                  // HH: first-stage values shared by a sweep's moves (absent if memory is short)
+    void* st1 = nullptr;                  // FP64 HH, RK4: first-stage values shared by a sweep's moves (stage1_buffer)
     unsigned* bar = nullptr;
     unsigned long long* flags = nullptr;  // neighbour epoch flags [2][kMaxGrid] of the sweep kernel
     uint64_t epoch = 0;                   // sweeps launched so far: the flags' epoch base
@@ -145,7 +145,7 @@ Ctx make_ctx(pimc_t h)
     c.fx = hh_fixed_of(h->dt);
     c.hRm = 0.5 * h->Rm;
     for (int a = 0; a < 4; ++a) c.hRf[a] = 0.5 * h->Rf[a];
-    c.st1 = h->st1;
+    c.st1 = (int64_t*)h->st1;
     return c;
 }
 
@@ -324,6 +324,27 @@ void choose_grid(pimc_t h)
                   h->grid <= sweep_max_grid(h->model, h->prec, h->device, 1);
 }
 
+// The first-stage values that a sweep's parameter moves share: held by handles
+// that use them (FP64 HH under the RK4 scheme, once they have data), given back
+// when the precision leaves FP64.  A cache only: without it (memory short) every
+// move evaluates the whole map.
+void stage1_buffer(pimc_t h)
+{
+    if (h->model == PIMC_MODEL_HH && h->prec == PIMC_FP64 && h->scheme == PIMC_SCHEME_RK4 && h->have_data && !h->st1) {
+        if (cudaMalloc(&h->st1, sizeof(int64_t) * 5 * h->ldx) != cudaSuccess) {
+            cudaGetLastError();
+            h->st1 = nullptr;
+            return;
+        }
+        h->ctx_version++;
+    } else if (h->st1 && h->prec != PIMC_FP64) {
+        cudaStreamSynchronize(h->stream);
+        cudaFree(h->st1);
+        h->st1 = nullptr;
+        h->ctx_version++;
+    }
+}
+
 int check_finite(const double* v, int64_t n)
 {
     for (int64_t i = 0; i < n; ++i)
@@ -442,11 +463,6 @@ int pimc_create(pimc_t* out, int model, int64_t M, int D, int L, double dt, cons
             return r;
         }
     }
-    // a cache only: without it every move evaluates the whole map
-    if (model == PIMC_MODEL_HH && cudaMalloc(&h->st1, sizeof(int64_t) * 5 * h->ldx) != cudaSuccess) {
-        cudaGetLastError();
-        h->st1 = nullptr;
-    }
     // zeroed on the handle's stream, ahead of everything launched on it
     cudaMemsetAsync(h->bar, 0, sizeof(unsigned) * 4, h->stream);
     cudaMemsetAsync(h->halo, 0, sizeof(unsigned long long) * 2 * kMaxResidentGrid * 8, h->stream);
@@ -514,6 +530,7 @@ int pimc_set_precision(pimc_t h, int precision)
     if ((r = put_rows(h, h->sig, S.data())) != PIMC_OK) return r;
     if (h->have_data && (r = convert_data(h)) != PIMC_OK) return r;
     choose_grid(h);
+    stage1_buffer(h);
     return refresh(h);
 }
 
@@ -523,6 +540,7 @@ int pimc_set_scheme(pimc_t h, int scheme)
     if (scheme != PIMC_SCHEME_RK4 && scheme != PIMC_SCHEME_TRAPEZOID) return fail(h, PIMC_ERR_ARG, "unknown scheme %d", scheme);
     h->scheme = scheme;
     h->ctx_version++;
+    stage1_buffer(h);
     return refresh(h);
 }
 
@@ -544,6 +562,7 @@ int pimc_set_data(pimc_t h, const double* y, const double* I_inj)
     int r = upload_data(h, y, I_inj);
     if (r != PIMC_OK) return r;
     h->have_data = true;
+    stage1_buffer(h);
     CK(h, launch_init_path(h->model, h->prec, make_ctx(h), h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     return refresh(h);
@@ -1395,6 +1414,7 @@ extern "C" int pimc_checkpoint_load(pimc_t h, const char* path)
     h->ctx_version++;
     CK(h, cudaMemsetAsync(h->bar, 0, sizeof(unsigned) * 4, h->stream));
     choose_grid(h);
+    stage1_buffer(h);
     return push_state(h);
 }
 

@@ -1205,7 +1205,7 @@ __device__ __forceinline__ bool param_terms_fixed(const Ctx& c, const Coef<doubl
 {
     const double* X = (const double*)c.X;
     const double* I = (const double*)c.I;
-    int64_t* st1 = (int64_t*)c.st1;
+    int64_t* st1 = c.st1;
     const HhFixedParams P = hh_fixed_params(c.fx, pq, k.dt);
     for (int64_t n = n0 + threadIdx.x; n < nend; n += NT) {
         if (!chk_site(c, 2, n)) continue;
