@@ -6,18 +6,20 @@
 // A parameter move (Sec. 4.3) needs the whole path: every CTA evaluates the
 // map at the proposed p for its sites into the inactive half of the
 // double-buffered cache and a partial change of action, summed exactly (integer
-// chunks, see "exact sums" below); after one grid barrier every CTA reads the
-// same total and takes the same accept decision, so no second launch or
-// broadcast is needed.  In FP32 the HH map of a parameter move runs on packed
-// f32x2 arithmetic: two adjacent sites a thread in the general form, the two
-// speculative outcomes of a site in the resident form.
+// chunks, see "exact sums" below); the CTAs' sums meet in words that carry their
+// own count and that every CTA polls ("counted sums"; under the trapezoid rule's
+// general form and in split chains of a batch: in accumulator slots read after a
+// grid barrier), so every CTA has the same total and takes the same accept
+// decision without a second launch or broadcast.  In FP32 the HH map of a
+// parameter move runs on packed f32x2 arithmetic: two adjacent sites a thread in
+// the general form, the two speculative outcomes of a site in the resident form.
 //
 // Two forms of the site phases:
 //  * resident (tiles of at most NT - 32 sites): thread 32 + i owns site
 //    n0 + i for the whole launch and keeps its operands in registers; the
 //    tile's neighbours are exchanged through shared memory and the two halo
-//    sites through global memory, ordered by epoch flags between neighbouring
-//    CTAs instead of grid barriers.  Warp 0 draws, reduces, synchronises and
+//    sites as packets of value and epoch in global memory, polled by the
+//    neighbouring CTA that needs them.  Warp 0 draws, reduces, synchronises and
 //    decides; while it waits for the other CTAs, the site threads evaluate the
 //    next parameter move's map for both outcomes of the pending decision.
 //  * general (any tile): threads stride over the tile, operands are read from
@@ -163,12 +165,12 @@ __device__ bool grid_barrier(const Ctx& c, int* s_abort, unsigned* phase, int ra
     return !*s_abort;
 }
 
-// Epoch flags between neighbouring CTAs (resident form).  After its sites of
-// parity ph have moved in the sweep with epoch e, a CTA stores e into
-// flags[ph][b] with a release store (after a CTA barrier, so it publishes the
-// CTA's writes); a neighbour polls, bounded, with acquire loads until the flag
-// reaches e.  Epochs only grow over a handle's launches (the host passes the
-// base in c.ep0).
+// Epoch flags between neighbouring CTAs (general form of a chain's own launch).
+// After its even sites have moved in the sweep with epoch e (ph 0), and at the
+// sweep's end (ph 1), a CTA stores e into flags[ph][b] with a release store (after
+// a CTA barrier, so it publishes the CTA's writes); a neighbour polls, bounded,
+// with acquire loads until the flag reaches e.  Epochs only grow over a handle's
+// launches (the host passes the base in c.ep0).
 __device__ __forceinline__ void flag_post(const Ctx& c, int ph, unsigned long long e)
 {
     if ((int)blockIdx.x == c.skip_cta) return;
