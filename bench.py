@@ -753,6 +753,14 @@ def run_ess(args):
     return res
 
 
+def emit(line, studies):
+    """The bench line alone on standard output, short enough for whoever keeps only the end of it; the default run's
+    studies (some 30 KB) as one JSON line on standard error."""
+    if studies:
+        print(json.dumps({"studies": studies}), file=sys.stderr, flush=True)
+    print(json.dumps(line), flush=True)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -986,8 +994,7 @@ def main():
                 "steady_state": steady, "fp64": fp64,
                 "rk4_maps_per_s": world * maps * NSKIP / (ms_per_step * 1e-3),
                 "param_moves_per_s": world * n_free * NSKIP / (ms_per_step * 1e-3)}
-        line.update(extras)
-        print(json.dumps(line))
+        emit(line, extras)
     if dist is not None:
         dist.destroy_process_group()
 
