@@ -17,8 +17,8 @@
 // Measured: the FP64 map is some 650 FP64 instructions, 49 000 scheduler cycles a warp; this one 5 300 with four warps a
 // scheduler and 9 100 alone (integer ALU and multiply-add pipes together; latency alone).  FP64 sweeps: M = 1000, 3 free
 // parameters, 120 -> 42 us; M = 32768, 7 free, 341 -> 97 us.  Of these the formats that follow a gate's range and the
-// FP64 additions cost 2 %, and the Jacobians' normalised products 7 % of an FP64 leapfrog step (M = 16384: 2435 ->
-// 2607 us for four trajectories of 20 steps).  Normals by the FP64 functions: some 90 FP64 instructions each; here 350
+// FP64 additions cost 2 %, and the Jacobians' normalised products 5 % of an FP64 leapfrog step (M = 16384: 2437 ->
+// 2570 us for four trajectories of 20 steps).  Normals by the FP64 functions: some 90 FP64 instructions each; here 350
 // cycles, of which the relative precision next to zeros costs 1 % of a sweep at M = 1000 (absolute formats: 5e-16 of a
 // normal's size, rms, where FP64 has 9e-17).
 //
@@ -245,16 +245,25 @@ PIMC_HD Fxn fx_norm(int64_t v, int f)
     const int lz = fx_clz32(h | 1u) - 1;
     return {(int64_t)fx_shl((uint64_t)v, lz), f + lz};
 }
-// From a double (zero for a subnormal one).
+// From a double (zero below 2^-200: products of a few factors stay far from FP64's smallest exponent).
 PIMC_HD Fxn fx_norm_of(double v)
 {
     const uint64_t b = fx_bits(v);
     const int ex = (int)((b >> 52) & 0x7ffu);
-    const int64_t m = ex ? (int64_t)(((b & 0xfffffffffffffull) | 0x10000000000000ull) << 10) : 0;
+    const int64_t m = ex >= 823 ? (int64_t)(((b & 0xfffffffffffffull) | 0x10000000000000ull) << 10) : 0;
     return {(b >> 63) ? -m : m, 1085 - ex};
 }
-PIMC_HD Fxn fx_fmul(const Fxn& a, const Fxn& b) { return {fx_smul<true>(a.m, b.m) * 2, a.f + b.f - 63}; }
+// (Not centred: a factor of zero gives zero.)
+PIMC_HD Fxn fx_fmul(const Fxn& a, const Fxn& b) { return {fx_smul(a.m, b.m) * 2, a.f + b.f - 63}; }
 PIMC_HD double fx_double(const Fxn& a) { return fx_double(a.m, a.f); }
+// m 2^-f as a double by the conversion instruction (its pipe is idle where this is used: 2596 -> 2570 us for the above).
+PIMC_HD double fx_double_conv(int64_t m, int f)
+{
+    const uint64_t b = fx_bits((double)m);
+    return fx_from_bits(m == 0 ? 0ull : b - ((uint64_t)(int64_t)f << 52));
+}
+// a b as a double.
+PIMC_HD double fx_dmul(const Fxn& a, const Fxn& b) { return fx_double_conv(fx_smul(a.m, b.m), a.f + b.f - 64); }
 
 // ---- 2^-y, 1/d -------------------------------------------------------------------------------------------------------
 
@@ -614,15 +623,15 @@ PIMC_HD bool hh_fixed_stage_adj(const HhFixed& c, const HhFixedParams& p, int64_
     const int64_t m2 = fx_smul(s[0], s[0]) * 4, mh = fx_smul(s[0], s[1]) * 4, n2 = fx_smul(s[2], s[2]) * 4;  // format 62
     const bool ok = hh_fixed_current(p, I46, V, fx_smul<true>(m2, mh), fx_smul<true>(n2, n2), K);
     const Fxn vNa = fx_norm(V - p.ENa, 55), vK = fx_norm(V - p.EK, 55), vL = {V - p.EL, 55};
-    const Fxn mm = fx_fmul(sn[0], sn[0]), m3 = fx_fmul(mm, sn[0]), vmm = fx_fmul(vNa, mm), vm3 = fx_fmul(vmm, sn[0]);
-    const Fxn nn = fx_fmul(sn[2], sn[2]), n3 = fx_fmul(nn, sn[2]), vn3 = fx_fmul(vK, n3);
-    const Fxn gm = fx_fmul(kNa, fx_fmul(vmm, sn[1])), gn = fx_fmul(kK, vn3);
-    const double dNa = fx_double(fx_fmul(p.kap, fx_fmul(vm3, sn[1]))), dK = fx_double(fx_fmul(p.kap, fx_fmul(vn3, sn[2])));
-    const double dL = fx_double(fx_fmul(p.kap, vL));
-    const double eNa = fx_double(fx_fmul(kNa, fx_fmul(m3, sn[1]))), eK = fx_double(fx_fmul(kK, fx_fmul(n3, sn[2])));
-    J[(kJg + 0) * stride] = fx_double((gm.m >> 2) * 3, gm.f - 2);
-    J[(kJg + 1) * stride] = fx_double(fx_fmul(kNa, vm3));
-    J[(kJg + 2) * stride] = fx_double(gn.m, gn.f - 2);
+    const Fxn mm = fx_fmul(sn[0], sn[0]), m3 = fx_fmul(mm, sn[0]), m3h = fx_fmul(m3, sn[1]);
+    const Fxn nn = fx_fmul(sn[2], sn[2]), n3 = fx_fmul(nn, sn[2]), n4 = fx_fmul(n3, sn[2]);
+    const Fxn kvNa = fx_fmul(kNa, vNa), kvK = fx_fmul(kK, vK);
+    const Fxn gm = fx_fmul(kvNa, fx_fmul(mm, sn[1]));
+    const double dNa = fx_dmul(fx_fmul(p.kap, vNa), m3h), dK = fx_dmul(fx_fmul(p.kap, vK), n4), dL = fx_dmul(p.kap, vL);
+    const double eNa = fx_dmul(kNa, m3h), eK = fx_dmul(kK, n4);
+    J[(kJg + 0) * stride] = fx_double_conv((gm.m >> 2) * 3, gm.f - 2);
+    J[(kJg + 1) * stride] = fx_dmul(kvNa, m3);
+    J[(kJg + 2) * stride] = fx_dmul({kvK.m, kvK.f - 2}, n3);
     J[(kJp + 0) * stride] = dNa;
     J[(kJp + 1) * stride] = dK;
     J[(kJp + 2) * stride] = dL;

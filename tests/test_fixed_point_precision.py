@@ -149,3 +149,22 @@ def test_draws_are_as_exact_as_fp64(lib, where):  # noqa: F811
         err, err64 = (g - x) / x, (y - x) / x
         assert _rms(err) <= 1.25 * _rms(err64)
         assert np.abs(err).max() <= np.abs(err64).max() + 2.0 ** -53
+
+
+@pytest.mark.parametrize("tiny", [0.0, 5e-324, 1e-300, -1e-150, 1e-80, -1e-40, 1e-19])
+def test_adjoint_at_vanishing_gates(lib, tiny):  # noqa: F811
+    """Gates of no size to speak of (and a drive of none): their Jacobian is that of gates at zero, to 2^-50 of a unit
+    entry, the gates' own scale."""
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+    out = []
+    for v in (tiny, 0.0):
+        for which in range(4):
+            x = np.array([[-65.0, 0.05, 0.6, 0.32]])
+            x[0, 1 + which % 3 if which < 3 else slice(1, 4)] = v
+            q, I, w = np.append(NOMINAL, 1.0)[None].copy(), np.array([v]), np.array([[1.0, 2.0, -1.0, 0.5]])
+            f, gx, gp, ok = np.zeros((1, 4)), np.zeros((1, 4)), np.zeros((1, 7)), np.zeros(1, dtype=np.uint8)
+            lib.adjoint(ctypes.c_double(0.02), p(q), p(x), p(I), p(w), ctypes.c_long(1), p(f), p(gx), p(gp), p(ok))
+            assert ok[0]
+            out.append(np.concatenate([f[0], gx[0], gp[0]]))
+    a, b = np.array(out[:4]), np.array(out[4:])
+    assert np.all(np.abs(a - b) <= 2.0 ** -50 * np.maximum(1.0, np.abs(b)))
