@@ -63,10 +63,23 @@ __global__ void load_refresh_kernel(Ctx c, const double* y64, const double* I64,
 }
 
 // Path element (a, n) from either the handle's storage or a dense FP64 array.
-template <class R>
-__device__ __forceinline__ R path_at(const Ctx& c, const double* Xe, int a, int64_t n)
+// x_n of the path in Xe (dense FP64 rows) or of the handle: every load ahead of
+// the first conversion, whose branch for values out of FP32's normal range waits
+// for its operand (one load after the other, FP32-mixed HH: action M = 16384 10.3
+// us, gradient M = 10^6 99; so 9.0 and 92).
+template <class R, int D>
+__device__ __forceinline__ void path_load(const Ctx& c, const double* Xe, int64_t n, R* x)
 {
-    return Xe ? narrow<R>(Xe[a * (c.M + 1) + n]) : ((const R*)c.X)[a * c.ldx + n];
+    if (Xe) {
+        double w[D];
+#pragma unroll
+        for (int a = 0; a < D; ++a) w[a] = Xe[a * (c.M + 1) + n];
+#pragma unroll
+        for (int a = 0; a < D; ++a) x[a] = narrow<R>(w[a]);
+    } else {
+#pragma unroll
+        for (int a = 0; a < D; ++a) x[a] = ((const R*)c.X)[a * c.ldx + n];
+    }
 }
 
 // A = A_o + A_f (beta = 1): out = (A, A_o, A_f).  Per-site residuals in R,
@@ -84,16 +97,37 @@ __global__ void __launch_bounds__(kBlock) action_kernel(Ctx c, const double* Xe,
     double v[2] = {0.0, 0.0};
     const R* y = (const R*)c.y;
     for (int64_t n = (int64_t)blockIdx.x * kBlock + threadIdx.x; n <= c.M; n += (int64_t)gridDim.x * kBlock) {
-        R x[D];
-        for (int a = 0; a < D; ++a) x[a] = path_at<R>(c, Xe, a, n);
+        const bool next = n < c.M;
+        const R yn = n >= 1 ? y[n] : R(0);
+        // x_n and, but at the last site, x_{n+1}: every load ahead of the first
+        // conversion (path_load)
+        R x[D], x1[D];
+        if (Xe) {
+            double w[D], w1[D];
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+                w[a] = Xe[a * (c.M + 1) + n];
+                w1[a] = next ? Xe[a * (c.M + 1) + n + 1] : 1.0;
+            }
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+                x[a] = narrow<R>(w[a]);
+                x1[a] = narrow<R>(w1[a]);
+            }
+        } else {
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+                x[a] = ((const R*)c.X)[a * c.ldx + n];
+                x1[a] = next ? ((const R*)c.X)[a * c.ldx + n + 1] : R(1);
+            }
+        }
         if (n >= 1) {
-            const R d = x[0] - y[n];
-            const double dd = widen(d);
+            const double dd = widen(R(x[0] - yn));
             v[0] += c.hRm * dd * dd;
         }
-        if (n < c.M) {
-            R g[D], g1[D], x1[D];
-            for (int a = 0; a < D; ++a) { x1[a] = path_at<R>(c, Xe, a, n + 1); g1[a] = R(0); }
+        if (next) {
+            R g[D], g1[D];
+            for (int a = 0; a < D; ++a) g1[a] = R(0);
             cache_value<Model, R>(c, kc, x, pr, n, g);
             if (c.scheme != kSchemeRK4) cache_value<Model, R>(c, kc, x1, pr, n + 1, g1);
             for (int a = 0; a < D; ++a) {
@@ -144,10 +178,18 @@ __global__ void __launch_bounds__(kBlock) grad_kernel(Ctx c, const double* Xe, c
         const int64_t n0 = tile * T, k = n0 - 1 + i;
         const bool has_x = i <= T && k >= 0 && k <= c.M, term = i <= T && k >= 0 && k < c.M;
         const bool owner = i >= 1 && i <= T && k <= c.M;
-        if (has_x)
-            for (int a = 0; a < D; ++a) xs[a][i] = path_at<R>(c, Xe, a, k);
-        if (i == 0 && n0 + T <= c.M)
-            for (int a = 0; a < D; ++a) xs[a][T + 1] = path_at<R>(c, Xe, a, n0 + T);
+        if (has_x) {
+            R x[D];
+            path_load<R, D>(c, Xe, k, x);
+#pragma unroll
+            for (int a = 0; a < D; ++a) xs[a][i] = x[a];
+        }
+        if (i == 0 && n0 + T <= c.M) {
+            R x[D];
+            path_load<R, D>(c, Xe, n0 + T, x);
+#pragma unroll
+            for (int a = 0; a < D; ++a) xs[a][T + 1] = x[a];
+        }
         __syncthreads();
         R own[D];
         for (int a = 0; a < D; ++a) own[a] = R(0);
