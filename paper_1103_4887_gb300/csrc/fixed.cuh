@@ -8,19 +8,20 @@
 // A value a in "format f" is the integer a 2^f.  Every intermediate has a range that the checks below guarantee: a
 // state, parameter, drive or step outside it makes hh_map_fixed return false, and the caller evaluates the FP64 map
 // instead (per lane).  In range, the map is as exact as the same formulas in FP64: its rms error against extended
-// precision was 0.97 to 1.01 times FP64's in V, and in every binade of a gate's result from 1 down to 2^-13 at most 1.12
+// precision was 0.5 to 1.01 times FP64's in V, and in every binade of a gate's result from 1 down to 2^-13 at most 1.12
 // times it (h deep in a spike), mostly less than it; the last addition of a gate is FP64's own, so that small gates keep
-// their bits.  The stages' Jacobians keep a relative precision of FP64's, whatever their size: below threshold d/dgNa is off
-// by 1.2e-16 of its rms, d/dm by 1.2e-16, d/dC (net currents of 0.1 out of 10) by 2e-14, as with FP64 instructions; in
-// absolute formats of 50 to 60 bits they were off by 4.7e-14, 1.5e-15 and 4.1e-13.
+// their bits.  The stages' Jacobians keep a relative precision of FP64's, whatever their size: below threshold d/dgNa is
+// off by 1.2e-16 of its rms, d/dm by 1.2e-16, d/dC (net currents of 0.1 out of 10) by 2e-14, as with FP64 instructions;
+// in absolute formats of 50 to 60 bits they were off by 4.7e-14, 1.5e-15 and 4.1e-13.
 //
-// Measured: the FP64 map is some 650 FP64 instructions, 49 000 scheduler cycles a warp; this one 5 300 with four warps a
-// scheduler and 9 100 alone (integer ALU and multiply-add pipes together; latency alone).  FP64 sweeps: M = 1000, 3 free
-// parameters, 120 -> 42 us; M = 32768, 7 free, 341 -> 97 us.  Of these the formats that follow a gate's range and the
-// FP64 additions cost 2 %, and the Jacobians' normalised products 5 % of an FP64 leapfrog step (M = 16384: 2437 ->
-// 2570 us for four trajectories of 20 steps).  Normals by the FP64 functions: some 90 FP64 instructions each; here 350
-// cycles, of which the relative precision next to zeros costs 1 % of a sweep at M = 1000 (absolute formats: 5e-16 of a
-// normal's size, rms, where FP64 has 9e-17).
+// Measured: the FP64 map is some 650 FP64 instructions, 49 000 scheduler cycles a warp; this one 6 460 with two warps a
+// scheduler (6.2e9 maps/s; 6 200 with absolute formats of 59 and 60 bits) and some 9 000 alone: integer ALU and
+// multiply-add pipes together, or latency alone.  FP64 sweeps: M = 1000, 3 free parameters, 120 -> 43 us; a pass of 20
+// sweeps at M = 32768, 7 free, 7.7 -> 2.06 ms.  Of these the formats that follow a gate's range and the FP64 additions
+// cost 2 %, and the Jacobians' normalised products 5 % of an FP64 leapfrog step (M = 16384: 2437 -> 2570 us for four
+// trajectories of 20 steps).  Normals by the FP64 functions: some 90 FP64 instructions each; here 350 cycles, of which
+// the relative precision next to zeros costs 1 % of a sweep at M = 1000 (absolute formats: 5e-16 of a normal's size, rms,
+// where FP64 has 9e-17).
 //
 // Integer arithmetic gives the same bits in every kernel and on the host, so the file also compiles as plain C++.
 #pragma once

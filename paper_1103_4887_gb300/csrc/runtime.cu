@@ -211,18 +211,23 @@ constexpr int64_t kDeviceRows = 65536;
 
 // Writes one byte of every page of a pageable buffer that a copy is about to
 // fill: pages not yet mapped would be faulted in by the device, one by one
-// (512 reads of 16..130 KB: 105 -> 133 ms).  Page-locked memory is mapped, and it
-// may be the source of an upload still waiting on the stream (pimc_load_data's
-// arrays are the caller's again only after this call's synchronisation): left
-// alone.
+// (512 reads of 16..130 KB: 105 -> 133 ms).
 void touch(void* p, size_t bytes)
+{
+    volatile char* c = (volatile char*)p;
+    for (size_t i = 0; i < bytes; i += 4096) c[i] = 0;
+    if (bytes) c[bytes - 1] = 0;
+}
+
+// The same for a caller's buffer.  Page-locked memory is mapped, and it may be the
+// source of an upload still waiting on the stream (pimc_load_data's arrays are the
+// caller's again only after this call's synchronisation): left alone.
+void touch_callers(void* p, size_t bytes)
 {
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) cudaGetLastError();
     else if (at.type != cudaMemoryTypeUnregistered) return;
-    volatile char* c = (volatile char*)p;
-    for (size_t i = 0; i < bytes; i += 4096) c[i] = 0;
-    if (bytes) c[bytes - 1] = 0;
+    touch(p, bytes);
 }
 
 int get_rows(pimc_t h, double* dst, const void* src, int64_t ld, bool state = false)
@@ -230,11 +235,11 @@ int get_rows(pimc_t h, double* dst, const void* src, int64_t ld, bool state = fa
     const int64_t n1 = h->M + 1, n = h->D * n1;
     std::unique_ptr<float[]> t;
     if (h->prec == PIMC_FP64) {
-        touch(dst, sizeof(double) * n);
+        touch_callers(dst, sizeof(double) * n);
         CK(h, cudaMemcpy2DAsync(dst, sizeof(double) * n1, src, sizeof(double) * ld, sizeof(double) * n1, h->D,
                                 cudaMemcpyDeviceToHost, h->stream));
     } else if (n >= kDeviceRows) {
-        touch(dst, sizeof(double) * n);
+        touch_callers(dst, sizeof(double) * n);
         CK(h, launch_rows_out(h->prec, src, ld, h->D, n1, h->dense, h->stream));
         CK(h, cudaMemcpyAsync(dst, h->dense, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
     } else {
@@ -278,7 +283,7 @@ int get_moments(pimc_t h, const double* S1, const double* S2, const double* shif
         for (int v = 0; v < 2; ++v) {
             double* dst = v == 0 ? mean : var;
             if (!dst) continue;
-            touch(dst + i, sizeof(double) * k);
+            touch_callers(dst + i, sizeof(double) * k);
             CK(h, launch_moments(S1 + i, S2 + i, sh, k, J, v == 0 ? h->dense : nullptr, v == 0 ? nullptr : h->dense,
                                  h->stream));
             CK(h, cudaMemcpyAsync(dst + i, h->dense, sizeof(double) * k, cudaMemcpyDeviceToHost, h->stream));
